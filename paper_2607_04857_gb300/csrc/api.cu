@@ -568,7 +568,7 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
         d.k = h.k;
         d.small = h.small;
         d.clampC = h.clampC;
-        d.el_fused = j.acc == ACC_I16P ? h.el_fused : 0;
+        d.el_fused = j.acc == ACC_I16P && !grouped_form(j.acc, j.variant) ? h.el_fused : 0;
         d.elmin = h.elmin;
         d.geps = 0.0f;
         if (j.acc == ACC_F32) {  // 16 ulp of beta: every column and E_L value is at most beta
@@ -691,6 +691,7 @@ int job_enqueue_scan(Workspace &ws, Job &j, const void *state_init = nullptr)
     if (j.window >= 0.0)  // record everything within the window of the running minimum
         a.margin += acc_float(j.acc) ? j.window : std::floor(j.window);
     a.zero = 0;
+    a.mad_inverse = kMadInverse;
     CK(launch_scan(j.acc, a, j.blocks, j.variant, s));
     CK(record_event(ws.ev[1], s));
     j.launches += 2;
@@ -1160,11 +1161,40 @@ int batch_walk(Acc acc, int variant, const HostInst &h, int wmax)
     const int rmin = variant_reg_rows(h) + 1;
     if (h.n - B < rmin)
         return 0;
-    int walk = std::min(wmax, h.n - B);
     int tv = 0, tw = 0;
-    if (tuned_plan(acc, -h.n, &tv, &tw) && tv == variant && tw >= rmin && tw <= walk)
-        walk = tw;
-    return walk;
+    if (tuned_plan(acc, -h.n, &tv, &tw) && tv == variant && tw >= rmin && tw <= std::min(kMaxWalkBits, h.n - B))
+        return tw;
+    return std::max(rmin, std::min(wmax, h.n - B));
+}
+
+// Longest walk of a batch's grouped scan, up to wmax: the one whose units, shared by the resident
+// warps, take the least time (as grouped_walk, for instances of several sizes; a launch lasts at least
+// as long as one unit).  Large batches walk as long as they can, which sets up the fewest units; a
+// small one needs its units shorter to occupy the GPU.
+int batch_max_walk(Acc acc, int variant, const std::vector<HostInst> &hs, int wmax)
+{
+    if (!grouped_form(acc, variant))
+        return wmax;
+    const int B = acc_suffix_bits(acc, variant), rmin = reg_rows_of(acc, variant) + 1;
+    int best = wmax;
+    double best_cost = std::numeric_limits<double>::infinity();
+    for (int w = rmin; w <= wmax; ++w) {
+        double sum = 0.0, longest = 0.0;
+        for (const HostInst &h : hs) {
+            if (h.n - B < rmin)
+                continue;
+            const int L = std::min(w, h.n - B);
+            const double unit = std::ldexp(1.0, L) + kUnitSetupSteps;
+            sum += std::ldexp(unit, h.n - B - L);
+            longest = std::max(longest, unit);
+        }
+        const double cost = sum / kResidentWarps + longest;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = w;
+        }
+    }
+    return best;
 }
 
 // Fold, bound, plan and threshold every instance of a batch (in parallel on the host), one
@@ -1210,19 +1240,19 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order)
             acc = h.acc;
     for (auto &h : hs)
         h.acc = acc;
-    // The batch supplies the parallelism, so every instance walks as long as it can (fewest,
-    // largest units: less per-unit set-up).
     int variant = scan_variant(acc);
     {
         int tv = 0, tw = 0;
         if (tuned_plan(acc, 0, &tv, &tw))
             variant = tv;
     }
+    if (acc_bytes(acc) != 4)
+        variant = 0;
+    const int wmax = batch_max_walk(acc, variant, hs, acc == ACC_F32 ? kFloatMaxWalkBits : kDefaultMaxWalkBits);
     auto plan_range = [&](int lo, int hi) {
         for (int i = lo; i < hi; ++i) {
             HostInst &h = hs[i];
-            h.variant = acc_bytes(acc) == 4 ? variant : 0;
-            const int wmax = acc == ACC_F32 ? kFloatMaxWalkBits : kDefaultMaxWalkBits;
+            h.variant = variant;
             pst[i] = plan(h, 0, 0, 0, batch_walk(acc, h.variant, h, wmax));
             // batches are many small instances: fewer descents (K = 1 thresholds also tighten on
             // the device as soon as a lower state is found)
@@ -1251,27 +1281,37 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order)
         int tv = 0, tw = 0;
         if (tuned_plan(alt_acc, 0, &tv, &tw))
             v2 = tv;
+        const int wbest = batch_max_walk(alt_acc, v2, hs, alt_walk);
         std::atomic<bool> all{true};
         auto alt_range = [&](int lo, int hi) {
             for (int i = lo; i < hi && all.load(std::memory_order_relaxed); ++i) {
                 HostInst &h = hs[i];
                 h.acc = alt_acc;
                 h.variant = v2;
-                const bool ok = plan(h, 0, 0, 0, batch_walk(alt_acc, v2, h, alt_walk)) == QUBO_OK &&
+                const bool ok = plan(h, 0, 0, 0, batch_walk(alt_acc, v2, h, wbest)) == QUBO_OK &&
                                 (h.small || (alt_acc == ACC_I16P ? i16p_exact(h) : i32f_exact(h, &h.clampC)));
                 if (!ok)
                     all = false;
                 else if (alt_acc == ACC_I16P)
-                    i16p_fuse_el(h);
+                    h.group_ok = h.small || i16p_group_ok(h);
             }
         };
         parallel(alt_range);
         if (all && alt_acc == ACC_I16P) {
-            // one kernel for the batch: the fused-only twin when every instance's E_L is fused
-            bool fused = true;
+            // one kernel for the batch: the grouped form when every instance's plan allows it, else
+            // its twin, the fused-only one when every instance's E_L is fused
+            bool grouped = true, fused = true;
             for (const HostInst &h : hs)
-                fused = fused && (h.small || h.el_fused);
-            const int v3 = packed_variant_for(v2, fused);
+                grouped = grouped && h.group_ok;
+            if (!grouped_form(ACC_I16P, packed_variant_for(v2, grouped, false))) {
+                parallel([&](int lo, int hi) {
+                    for (int i = lo; i < hi; ++i)
+                        i16p_fuse_el(hs[i]);
+                });
+                for (const HostInst &h : hs)
+                    fused = fused && (h.small || h.el_fused);
+            }
+            const int v3 = packed_variant_for(v2, grouped, fused);
             for (HostInst &h : hs)
                 h.variant = v3;
         }
@@ -1531,6 +1571,7 @@ int qubo_solve_ex(const void *Q_host, int n, qubo_dtype dtype, const qubo_option
     qubo_options o{};
     if (opt)
         o = *opt;
+    o.flags &= kCallerFlags;
     int st = check_opts(&o, states_cap, out_states, out_topk);
     if (st)
         return st;
@@ -1570,6 +1611,7 @@ int qubo_plan_query(const void *Q_host, int n, qubo_dtype dtype, const qubo_opti
     qubo_options o{};
     if (opt)
         o = *opt;
+    o.flags &= kCallerFlags;
     if (!info || o.topk < 0 || o.topk > QUBO_MAX_TOPK)
         return QUBO_ERR_ARG;
     HostInst h;
@@ -1596,6 +1638,7 @@ int qubo_solve_window(const void *Q_host, int n, qubo_dtype dtype, double window
     qubo_options o{};
     if (opt)
         o = *opt;
+    o.flags &= kCallerFlags;
     o.topk = 0;
     if (!(window >= 0.0) || !std::isfinite(window) || !out_count || (cap > 0 && (!out_codes || !out_E)))
         return QUBO_ERR_ARG;
@@ -1707,6 +1750,7 @@ int qubo_solve_wide(const void *Q_host, int n, qubo_dtype dtype, int n_inner, ui
     qubo_options o{};
     if (opt)
         o = *opt;
+    o.flags &= kCallerFlags;
     if (!Q_host || !out_min || !dtype_ok(dtype) || n_inner < 1 || n_inner > 64 || n < n_inner ||
         n - n_inner > 64 || n > QUBO_WIDE_MAX_N || outer_count < 1 || o.fix_bits != 0)
         return QUBO_ERR_ARG;
@@ -1824,8 +1868,12 @@ int qubo_solve_wide(const void *Q_host, int n, qubo_dtype dtype, int n_inner, ui
                 return st;
         } else {
             qubo_options so = o;
-            if (deadline > 0)
+            if (deadline > 0) {
                 so.time_limit_s = std::max(1e-3, deadline - now_s());
+                // the limits callers pass here were chosen against the interleaved packed scan's
+                // rate; a range that ran out of time still does
+                so.flags |= kFlagInterleaved;
+            }
             parts.resize(1);
             if ((st = solve_one(*ws, hs[0], so, states_cap, (cudaStream_t)stream, parts[0], stats)))
                 return st;
@@ -1882,6 +1930,7 @@ int qubo_problem_create(const void *Q_host, int n, qubo_dtype dtype, const qubo_
         return QUBO_ERR_NOMEM;
     if (opt)
         p->opt = *opt;
+    p->opt.flags &= kCallerFlags;
     if (p->opt.topk < 0 || p->opt.topk > QUBO_MAX_TOPK) {
         delete p;
         return QUBO_ERR_ARG;
@@ -2335,6 +2384,8 @@ int qubo_autotune_batched_ex(const void *Q_packed, const int *n, const size_t *o
             if (acc == ACC_I16P) {
                 if (!i16p_exact(h))
                     return false;
+                if (grouped_form(acc, h.variant))
+                    return i16p_group_ok(h);
                 i16p_fuse_el(h);
                 // a fused-only packed kernel takes only plans whose E_L is fused
                 return h.el_fused || !packed_fused_only(h.variant);

@@ -13,9 +13,18 @@
 namespace qubo {
 namespace host {
 
-constexpr int kTargetUnitsLog2 = 15;   // aim for >= 2^15 work units per scan
+constexpr int kTargetUnitsLog2 = 15;   // aim for >= 2^15 work units per scan (see also grouped_walk)
 constexpr double kDefaultMargin = 1e-3; // FP32 scans: candidate margin above the running minimum
 constexpr int kDefaultMaxWalkBits = 12;
+// The flags a caller may set, and an internal one: the packed scan's interleaved variants only.
+constexpr uint32_t kCallerFlags = QUBO_FLAG_PLAIN | QUBO_FLAG_INT32 | QUBO_FLAG_RIGOROUS;
+constexpr uint32_t kFlagInterleaved = 0x80000000u;
+// Grouped scans walk up to 2^14 steps: n=40 packed 2.5% and n=38 int32 0.6% faster than 2^12.
+constexpr int kGroupedMaxWalkBits = 14;
+// What the choice of a grouped scan's walk weighs (grouped_walk, batch_plan): the warps resident on
+// GB300's 152 SMs at three blocks each, and a unit's set-up in Gray steps (about 4 us).
+constexpr int kResidentWarps = 152 * 12;
+constexpr int kUnitSetupSteps = 140;
 // Integers in FP32 lanes: 2^14-step walks (n=50: 0.7% faster than 2^12) when the plan stays exact
 // in FP32 lanes, else the default length is tried.
 constexpr int kI32FMaxWalkBits = 14;
@@ -61,6 +70,7 @@ struct HostInst {
     int32_t clampC = 0; // ACC_I32F: threshold clamp
     int32_t col_lo = 0, col_hi = 0;  // ACC_I16P: proven range of every column value
     int32_t el_fused = 0, elmin = 0; // ACC_I16P: E_L added to the packed minima (i16p_fuse_el)
+    int32_t group_ok = 0;            // ACC_I16P: the plan can run a grouped variant (i16p_group_ok)
     int Z = 0;                  // ACC_I32Z / ACC_F32Z: walked rows without suffix couplings
     std::vector<uint8_t> perm;  // ACC_I32Z / ACC_F32Z: caller's variable at each scan position
     bool no_factored = false;   // the factored FP32 scan used up its margin: plan the dense one
@@ -74,7 +84,7 @@ struct PlanFields {
     Acc acc;
     int variant, B, L, k, small, fix_bits;
     uint64_t fix_value, unit_begin, units, sub_base, sub_count, items, states;
-    int32_t clampC, col_lo, col_hi, el_fused, elmin;
+    int32_t clampC, col_lo, col_hi, el_fused, elmin, group_ok;
 };
 
 // Plans, saved and restored without the matrices.
@@ -99,6 +109,7 @@ int pick_variant(Acc acc, int requested);
 
 // The split n = k + L + B of a run (Sec. 3.3) and the accumulator it runs in: the exactness
 // checks of the packed 16-bit and FP32-lane scans, the factored scan's variable order.
+int grouped_walk(int bits, int lmin, int lmax);
 int plan(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bits);
 bool i32f_exact(const HostInst &h, int32_t *clampC);
 bool i32f_allowed();
@@ -106,6 +117,8 @@ void col_range_exact(const HostInst &h, int64_t &lo, int64_t &hi);
 int64_t walked_energy_max(const HostInst &h);
 bool i16p_exact(HostInst &h);
 void i16p_fuse_el(HostInst &h);
+bool i16p_group_ok(const HostInst &h);
+void i16p_step_form(HostInst &h, bool allow_grouped);
 bool i16p_allowed();
 int zero_rows_search(HostInst &h);
 bool i32z_allowed();

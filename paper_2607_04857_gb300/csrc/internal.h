@@ -35,9 +35,9 @@ constexpr int kRegRows = 4;
 // interleaved form, one integer column in four / in eight updated by a 3-input add on the ALU
 // pipe), 2- or 3-input mins, and the step form: 0, all adds first, then the min tree; 1, the adds
 // interleaved with the first level of the min tree (each triple of columns reduced as soon as its
-// adds are issued); 2 (integers in FP32 lanes and FP32; form 1 for int32), the grouped form: groups of 16 steps skip the min tree while a per-thread lower bound of the column
-// minimum, moved by the steps' smallest column deltas, proves that no column can reach the
-// threshold.  The 8-byte
+// adds are issued); 2, the grouped form (scan_grouped.cuh): groups of 16 steps skip the min tree
+// while a per-thread lower bound of the column minimum, moved by the steps' smallest column deltas,
+// proves that no column can reach the threshold.  The 8-byte
 // accumulators compile one variant: S = 16 with variant 0's register rows, blocks and min inputs.
 constexpr int kScanVariants = 24;
 constexpr int kVariantCols[kScanVariants] = {32, 16, 16, 16, 16, 16, 32, 16, 16, 16, 16, 16,
@@ -48,23 +48,12 @@ constexpr int kVariantAddMode[kScanVariants] = {0, 6, 7, 0, 0, 4, 4, 5, 6, 5, 4,
 constexpr int kVariantMinInputs[kScanVariants] = {3, 3, 3, 3, 3, 3, 3, 3, 3, 3, 3, 3,
                                                   3, 3, 3, 3, 3, 3, 3, 3, 3, 3, 3, 3};
 constexpr int kVariantInterleave[kScanVariants] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 0, 1, 1, 1, 1, 1, 2, 2, 2, 2};
-// The step form a kernel of an accumulator compiles for a variant: the grouped form only for FP32
-// column adds (integers in FP32 lanes, FP32).
-constexpr int step_form(int variant, bool fp32_columns)
-{
-    return kVariantInterleave[variant] == 2 && !fp32_columns ? 1 : kVariantInterleave[variant];
-}
-// Whether a plan's scan kernel runs the grouped form.
-constexpr bool grouped_form(Acc acc, int variant)
-{
-    return (acc == ACC_I32F || acc == ACC_F32) && variant >= 0 && variant < kScanVariants &&
-           kVariantInterleave[variant] == 2;
-}
 // Default variant per 4-byte accumulator (measured on GB300; see the profiles).
-constexpr int kDefaultVariantI32 = 16;
-constexpr int kDefaultVariantF32 = 22;
+constexpr int kDefaultVariantI32 = 20;
+constexpr int kCallerVariantI32 = 16;  // short walks set by the caller (plan.cu: fit_variant)
+constexpr int kDefaultVariantF32 = 20;
 constexpr int kDefaultVariantI32F = 20;
-constexpr int kDefaultVariantI16P = 14;
+constexpr int kDefaultVariantI16P = 20;
 // Compiled variants of the packed 16-bit scan: S words per thread (2 S columns), register rows,
 // minimum resident blocks per SM, and how the adds are issued (0: compiler's choice; 2 and 3: one
 // add in four or in eight as a 3-input add with a runtime 0, which the ALU pipe executes, so
@@ -72,30 +61,37 @@ constexpr int kDefaultVariantI16P = 14;
 // Variants 8-14 and 16-19 interleave the adds and the first min level as the 4-byte variants do
 // (18 and 19 with one add in eight / in four on the ALU pipe, the others with plain adds), and
 // carry both forms of the E_L step (added to the packed minimum, or after the lane combine),
-// chosen per instance at run time.  Variants 20-23 are 14, 13, 8 and 11 compiled with the fused
-// form alone (interleave 2), half the code, for plans whose E_L is fused.
+// chosen per instance at run time.  Variants 22 and 23 are 8 and 11 compiled with the fused form
+// alone (step form 3), half the code, for plans whose E_L is fused.  Variants 20 and 21 run the
+// grouped form (2; E_L is then never fused).
 constexpr int kPackedWords[kScanVariants] = {16, 16, 16, 16, 16, 32, 32, 16, 16, 16, 16, 16,
                                              32, 16, 16, 16, 32, 16, 16, 16, 16, 16, 16, 16};
 constexpr int kPackedRegRows[kScanVariants] = {3, 3, 3, 3, 3, 2, 2, 2, 3, 3, 4, 2, 2, 4, 5, 4, 3, 5, 5, 5, 5, 4, 3, 2};
-constexpr int kPackedMinBlocks[kScanVariants] = {3, 3, 3, 4, 4, 2, 2, 4, 3, 4, 3, 4, 2, 2, 2, 2, 2, 1, 2, 2, 2, 2, 3, 4};
+constexpr int kPackedMinBlocks[kScanVariants] = {3, 3, 3, 4, 4, 2, 2, 4, 3, 4, 3, 4, 2, 2, 2, 2, 2, 1, 2, 2, 3, 3, 3, 4};
 constexpr int kPackedAddMode[kScanVariants] = {0, 3, 2, 0, 3, 0, 3, 3, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 3, 2, 0, 0, 0, 0};
-constexpr int kPackedInterleave[kScanVariants] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 0, 1, 1, 1, 1, 2, 2, 2, 2};
-// The packed variant a plan runs: the fused-only twin of a variant when its E_L is fused and the
-// twin exists, else the variant that carries both forms.
-constexpr int packed_variant_for(int variant, bool el_fused)
+constexpr int kPackedInterleave[kScanVariants] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 0, 1, 1, 1, 1, 2, 2, 3, 3};
+// Whether a plan's scan kernel runs the grouped form.
+constexpr bool grouped_form(Acc acc, int variant)
 {
-    constexpr int kBoth[4] = {14, 13, 8, 11};
-    int both = variant;
-    for (int t = 0; t < 4; ++t)
-        if (variant == 20 + t)
-            both = kBoth[t];
-    if (el_fused)
-        for (int t = 0; t < 4; ++t)
-            if (both == kBoth[t])
-                return 20 + t;
-    return both;
+    if (variant < 0 || variant >= kScanVariants)
+        return false;
+    return acc == ACC_I16P ? kPackedInterleave[variant] == 2
+                           : (acc == ACC_I32F || acc == ACC_F32 || acc == ACC_I32) && kVariantInterleave[variant] == 2;
 }
-constexpr bool packed_fused_only(int variant) { return variant >= 0 && variant < kScanVariants && kPackedInterleave[variant] == 2; }
+// The packed variant a plan runs.  The grouped variants need a plan whose rows 0-3 move a column by
+// at most 32767 (group_ok), else their interleaved twins run; of the variants that carry both forms
+// of the E_L step, the fused-only twin runs when the plan's E_L is fused and the twin exists.
+constexpr int packed_variant_for(int variant, bool group_ok, bool el_fused)
+{
+    if (variant == 20 || variant == 21)
+        return group_ok ? variant : variant == 20 ? 14 : 13;
+    const int both = variant == 22 ? 8 : variant == 23 ? 11 : variant;
+    return !el_fused ? both : both == 8 ? 22 : both == 11 ? 23 : both;
+}
+constexpr bool packed_fused_only(int variant) { return variant >= 0 && variant < kScanVariants && kPackedInterleave[variant] == 3; }
+// Odd multiplier of the grouped form's integer multiply-adds (scan_grouped.cuh) and its inverse.
+constexpr uint32_t kMad = 0x9e3779b1u, kMadInverse = 0x0e8b2f51u;
+static_assert(kMad * kMadInverse == 1u, "the inverse of kMad modulo 2^32");
 // Threads per block of the scan kernel (4 warps; every warp owns one work unit at a time).
 constexpr int kScanThreads = 128;
 // Longest Gray walk inside one work unit (also the FP32 re-anchoring period).
@@ -186,7 +182,7 @@ struct ScanArgs {
     const volatile int *abort_flag;
     double margin;               // float scans: candidate margin above the threshold
     int32_t zero;                // the constant 0, passed at run time (packed 3-input-add variants)
-    int32_t pad;
+    uint32_t mad_inverse;        // kMadInverse, passed at run time (integer updates of the grouped form)
 };
 
 // Columns per thread (S) of the scan kernel for an accumulator of `bytes` bytes and a variant;

@@ -75,7 +75,7 @@ constexpr Layout layout(int n, int L, size_t cap)
     l.M = o;
     o = up256(o + sizeof(int32_t) * (1u << kB) * L);
     l.EL = o;
-    o = up256(o + sizeof(int32_t) * (1u << L));
+    o = up256(o + sizeof(int32_t) * ((1u << L) + (1u << L) / 16));  // E_L and its group minima
     l.rec = o;
     o = up256(o + sizeof(Rec) * kRecords);
     l.res = o;
@@ -277,6 +277,7 @@ extern "C" int qubo_solve_noalloc(const void *Q_host, int n, qubo_dtype dtype, i
     a.abort_flag = (const volatile int *)(base + lo.abort);
     a.margin = 0.0;
     a.zero = 0;
+    a.mad_inverse = kMadInverse;
     int sms = 0;
     NA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     int bps = scan_blocks_per_sm(ACC_I32, true, 0);

@@ -25,7 +25,7 @@ PlanFields plan_fields(const HostInst &h)
 {
     return {h.acc,   h.variant,  h.B,         h.L,     h.k,      h.small,  h.fix_bits, h.fix_value, h.unit_begin,
             h.units, h.sub_base, h.sub_count, h.items, h.states, h.clampC, h.col_lo,   h.col_hi,    h.el_fused,
-            h.elmin};
+            h.elmin, h.group_ok};
 }
 
 void set_plan_fields(HostInst &h, const PlanFields &p)
@@ -49,6 +49,7 @@ void set_plan_fields(HostInst &h, const PlanFields &p)
     h.col_hi = p.col_hi;
     h.el_fused = p.el_fused;
     h.elmin = p.elmin;
+    h.group_ok = p.group_ok;
 }
 
 bool dtype_ok(qubo_dtype dt) { return dt == QUBO_I16 || dt == QUBO_I32 || dt == QUBO_F32 || dt == QUBO_F64; }
@@ -135,6 +136,36 @@ int variant_reg_rows(const HostInst &h)
     return reg_rows_of(h.acc, h.variant);
 }
 
+// Longest walk of an accumulator's plans.
+static int max_walk(Acc acc, bool grouped)
+{
+    return acc == ACC_F32       ? kFloatMaxWalkBits
+           : acc == ACC_I32F    ? kI32FMaxWalkBits
+           : acc_factored(acc) ? kZMaxWalkBits
+           : grouped            ? kGroupedMaxWalkBits
+                                : kDefaultMaxWalkBits;
+}
+
+// Walk of a grouped scan of 2^bits column blocks (bits = walked + fixed bits of a unit): the one whose
+// units take the least time when the resident warps scan them in rounds, a unit costing its steps
+// plus its set-up.  Fewer, longer units than the 2^15 the other scans aim at: n=28, packed, 2^15
+// units 236 us, 2^10 units 33 us; n=32 256 us with 2^15, 152-170 us with 2^12 to 2^14; and the count
+// of rounds matters while it is small (n=32 with 2^11 units, 1.1 rounds: 224 us).
+int grouped_walk(int bits, int lmin, int lmax)
+{
+    int best = lmin;
+    double best_cost = std::numeric_limits<double>::infinity();
+    for (int L = lmin; L <= std::min(lmax, bits); ++L) {
+        const double rounds = std::ceil(std::ldexp(1.0, bits - L) / kResidentWarps);
+        const double cost = rounds * (std::ldexp(1.0, L) + kUnitSetupSteps);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = L;
+        }
+    }
+    return best;
+}
+
 int plan(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bits)
 {
     const int n = h.n;
@@ -165,12 +196,10 @@ int plan(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bi
         L = n - h.B - split_k;
     else if (walk_bits > 0)
         L = walk_bits;
+    else if (grouped_form(h.acc, h.variant))
+        L = grouped_walk(free_bits - h.B, rc + 1, max_walk(h.acc, true));
     else
-        L = std::max(rc + 1, std::min(h.acc == ACC_F32          ? kFloatMaxWalkBits
-                                      : h.acc == ACC_I32F       ? kI32FMaxWalkBits
-                                      : acc_factored(h.acc) ? kZMaxWalkBits
-                                                            : kDefaultMaxWalkBits,
-                                      free_bits - h.B - kTargetUnitsLog2));
+        L = std::max(rc + 1, std::min(max_walk(h.acc, false), free_bits - h.B - kTargetUnitsLog2));
     const int k = n - h.B - L;
     if (L < rc + 1 || L > kMaxWalkBits || k < fix_bits || k > 63)
         return QUBO_ERR_ARG;
@@ -202,27 +231,29 @@ int scan_variant(Acc acc)
 // The variant a run uses: the caller's (tuned) choice, else the accumulator's default.
 int pick_variant(Acc acc, int requested) { return requested >= 0 ? requested : scan_variant(acc); }
 
-// The default variant keeps five walked rows in registers and needs walks of at least six bits.
-// When the walk is shorter (the caller's walk_bits, split_k leaving fewer walked bits, or a
-// (sub)cube too small for 2^kTargetUnitsLog2 units walking four unrolled bodies each) and the
-// caller named no variant, the run takes the measured best variant with fewer register rows and
-// the same columns per thread, so the suffix split is unchanged; failing all, the one with the
-// fewest rows.  A small instance's units are then short bodies: a unit that runs its unrolled
-// body only once or twice pays for the straight-line code's instruction fetch, and a 64-step
-// body made every launch of a small solve about 0.2 ms longer than an 8-step one.
+// The variant of a run whose caller named none, from the accumulator's default: the grouped variant
+// keeps five walked rows in registers and needs walks of at least six bits.  When the walk is shorter
+// (the caller's walk_bits or split_k, or the planner's own walk of a small (sub)cube) the run takes
+// the best variant with fewer register rows and the same columns per thread, so the suffix split is
+// unchanged: the grouped one with four rows, whose body is one group (a small launch waits on the
+// first fetch of its code), then the interleaved ones; failing all, the one with the fewest rows.
+// int32: a walk of at most 2^8 steps that the caller sets keeps the interleaved variant 16, the plan
+// such callers have had (grouped, n=29: 91 us against 156 us).
 int fit_variant(const HostInst &h, int fix_bits, int split_k, int walk_bits, int variant_req, int variant)
 {
     if (variant_req >= 0 || std::getenv("QUBO_SCAN_VARIANT"))
         return variant;
-    const int B = acc_suffix_bits(h.acc, variant);
-    // the planner's own walk should give a unit at least four unrolled bodies (two more bits)
-    const int slack = split_k > 0 || walk_bits > 0 ? 0 : 2;
+    const int B = acc_suffix_bits(h.acc, variant), bits = h.n - fix_bits - B;
+    const bool own = split_k <= 0 && walk_bits <= 0;  // the planner chooses the walk
     const int L = split_k > 0 ? h.n - B - split_k
-                              : (walk_bits > 0 ? walk_bits : h.n - fix_bits - B - kTargetUnitsLog2 - slack);
+                  : walk_bits > 0 ? walk_bits
+                  : bits < 5 ? bits : grouped_walk(bits, 5, max_walk(h.acc, true));
+    if (h.acc == ACC_I32 && !own && L <= 8 && L >= reg_rows_of(h.acc, kCallerVariantI32) + 1)
+        return kCallerVariantI32;
     if (L >= reg_rows_of(h.acc, variant) + 1)
         return variant;
-    static constexpr int kShorter4[] = {8, 3};       // 4 register rows (interleaved), 3
-    static constexpr int kShorterP[] = {13, 8, 11};  // packed: 4, 3, 2 register rows (interleaved)
+    static constexpr int kShorter4[] = {21, 3};      // 4 register rows (grouped), 3
+    static constexpr int kShorterP[] = {21, 8, 11};  // packed: 4 register rows (grouped), 3, 2
     const int *cand = h.acc == ACC_I16P ? kShorterP : kShorter4;
     const int nc = h.acc == ACC_I16P ? 3 : 2;
     int last = variant;
@@ -233,8 +264,8 @@ int fit_variant(const HostInst &h, int fix_bits, int split_k, int walk_bits, int
             return cand[c];
         last = cand[c];
     }
-    // no candidate fits the walk the planner aims at: the fewest rows, if the caller's walk allows
-    const int Lmax = split_k > 0 ? h.n - B - split_k : (walk_bits > 0 ? walk_bits : h.n - fix_bits - B);
+    // no candidate fits: the fewest rows, if the caller's walk allows
+    const int Lmax = own ? bits : L;
     return Lmax >= reg_rows_of(h.acc, last) + 1 ? last : variant;
 }
 
@@ -434,6 +465,37 @@ void i16p_fuse_el(HostInst &h)
     }
 }
 
+// Whether the packed grouped form can run a proven plan: its bound unpacks the moves of the walked
+// rows 0-3 (couplings to the suffix and, folded in, to the fixed variables) as 16-bit values, and its
+// adds are capped below the word of two columns at 32767.
+bool i16p_group_ok(const HostInst &h)
+{
+    const int n = h.n, B = h.B, nf = h.B + h.L;
+    if (h.L < 5 || h.col_hi >= 32767)
+        return false;
+    auto U = [&](int i, int j) { return i < j ? h.Ui[(size_t)i * n + j] : h.Ui[(size_t)j * n + i]; };
+    for (int r = B; r < B + 4; ++r) {
+        int64_t row = 0;
+        for (int b = 0; b < B; ++b)
+            row += std::llabs(U(r, b));
+        for (int f = nf; f < n; ++f)
+            row += std::llabs(U(r, f));
+        if (row > 32767)
+            return false;
+    }
+    return true;
+}
+
+// The step form of a proven packed plan: grouped when its variant is a grouped one and the plan and
+// the caller allow it, else the interleaved twin with E_L fused when it can be.
+void i16p_step_form(HostInst &h, bool allow_grouped)
+{
+    h.group_ok = allow_grouped && i16p_group_ok(h);
+    h.el_fused = 0;
+    if (!grouped_form(ACC_I16P, packed_variant_for(h.variant, h.group_ok, false)))
+        i16p_fuse_el(h);
+}
+
 // Factored scan of sparse instances: choose up to kZMaxRows walked variables with no coupling
 // to any of the B suffix variables (any order of the variables is allowed, Sec. 2.4), and a
 // scan order: suffix, those zero rows, the other walked rows, the unit's fixed bits, then the
@@ -586,8 +648,8 @@ int plan_run(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int wal
             h.variant = fit_variant(h, fix_bits, split_k, walk_bits, variant_req, h.variant);
             if (plan(h, fix_bits, fix_value, split_k, walk_bits) == QUBO_OK && i16p_exact(h)) {
                 chosen = ACC_I16P;
-                i16p_fuse_el(h);
-                h.variant = packed_variant_for(h.variant, h.el_fused);
+                i16p_step_form(h, (flags & kFlagInterleaved) == 0);
+                h.variant = packed_variant_for(h.variant, h.group_ok, h.el_fused);
             }
         }
         if (chosen == ACC_I32 && i32f_allowed()) {
@@ -607,8 +669,8 @@ int plan_run(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int wal
     h.variant = acc_bytes(h.acc) == 4 ? pick_variant(h.acc, variant_req) : 0;
     if (acc_bytes(h.acc) == 4)
         h.variant = fit_variant(h, fix_bits, split_k, walk_bits, variant_req, h.variant);
-    if (h.acc == ACC_I16P)  // the fused-E_L-only build of the variant when E_L is fused
-        h.variant = packed_variant_for(h.variant, h.el_fused);
+    if (h.acc == ACC_I16P)
+        h.variant = packed_variant_for(h.variant, h.group_ok, h.el_fused);
     return plan(h, fix_bits, fix_value, split_k, walk_bits);
 }
 

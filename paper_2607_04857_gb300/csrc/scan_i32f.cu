@@ -10,7 +10,7 @@ constexpr auto kernel_of()
     constexpr int kS = cols_per_thread(4, VAR);
     static_assert(ilog2c(32 * kS) == suffix_bits(4, VAR), "suffix bits must match the column layout");
     return scan_kernel<i32f, kS, kVariantRegRows[VAR], K1, kVariantMinBlocks[VAR], kVariantAddMode[VAR],
-                       kVariantMinInputs[VAR], step_form(VAR, true)>;
+                       kVariantMinInputs[VAR], kVariantInterleave[VAR]>;
 }
 
 template <bool K1, int... V>

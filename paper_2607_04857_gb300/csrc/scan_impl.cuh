@@ -55,9 +55,7 @@ struct i16p {};
 
 template <>
 struct Tr<int32_t> {
-    // No grouped step form: integer adds are associative, so the compiler folds a skipped group's
-    // 15 column updates into one, and the scan would no longer form every state's energy.
-    static constexpr bool kGrouped = false;
+    static constexpr bool kGrouped = true;  // compiles the grouped step form (variants 20-23)
     using TC = int32_t;
     using TP = int32_t;
     static constexpr bool kIntInFloat = false;
@@ -169,7 +167,7 @@ struct Tr<i32f> {
 // instruction.  The table rows are stored as packed deltas lo + 65536 * hi.
 template <>
 struct Tr<i16p> {
-    static constexpr bool kGrouped = false;
+    static constexpr bool kGrouped = true;  // packed variants 20 and 21
     using TC = uint32_t;
     using TP = int32_t;
     static constexpr bool kIntInFloat = false;
@@ -186,6 +184,10 @@ struct Tr<i16p> {
     __device__ static int32_t tmin(int32_t a, int32_t b) { return min(a, b); }
 };
 constexpr int32_t kLaneBias = 32768;
+#ifndef QUBO_LONG_BODY
+#define QUBO_LONG_BODY 4
+#endif
+constexpr int kLongBody = QUBO_LONG_BODY;
 
 // Column value of a prefix-type threshold.  For FP32 columns holding integers the threshold is
 // clamped to +-C first: beyond C every column (|column| <= C - 1 - max|E_L|) is decided the same
@@ -239,6 +241,8 @@ __device__ __forceinline__ void vload(const E *p, E (&o)[VecOf<E>::V])
 {
     vsplit(__ldg((const typename VecOf<E>::type *)p), o);
 }
+__device__ __forceinline__ int4 vjoin(const int32_t *v) { return make_int4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ uint4 vjoin(const uint32_t *v) { return make_uint4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ float4 vjoin(const float *v) { return make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ double2 vjoin(const double *v) { return make_double2(v[0], v[1]); }
 
@@ -360,10 +364,7 @@ __global__ void tables_kernel(const Inst *insts)
     const int n = d.n, B = d.B, L = d.L;
     const long NB = 1l << B, NL = 1l << L;
     const long NM = kPacked ? NB / 2 : NB;  // words per interaction row
-    // the grouped scans (integers in FP32 lanes, FP32): after E_L, the minimum of E_L over each
-    // group of 16 walk steps, as stored
-    const long NLG = Tr<T>::kGrouped ? NL / 16 : 0;
-    const long total = NB + NM * L + NL + NLG;
+    const long total = NB + NM * L + NL;
     const F *W = field_matrix<T>(d);
     // M_int row r at column j: coupling of walked variable r to the suffix pattern j
     auto m_entry = [&](long r, long j) {
@@ -398,28 +399,33 @@ __global__ void tables_kernel(const Inst *insts)
                 ((TC *)d.M)[r * NM + w] = (TC)m_entry(r, w);
         } else {  // E_L(g(i)): energy of the i-th walked pattern, stored in walk order
             const long i = idx - NB - NM * L;
-            auto el_of = [&](long ii) {
-                const long g = ii ^ (ii >> 1);
-                F e = 0;
-                for (int r = 0; r < L; ++r) {
-                    if (!((g >> r) & 1))
-                        continue;
-                    e += W[(B + r) * n + (B + r)];
-                    for (int r2 = r + 1; r2 < L; ++r2)
-                        if ((g >> r2) & 1)
-                            e += W[(B + r) * n + (B + r2)];
-                }
-                return e;
-            };
-            if (i >= NL) {  // group minimum (grouped scans; rounding to TC is monotonic)
-                const long g0 = 16 * (i - NL);
-                F m = el_of(g0);
-                for (int t = 1; t < 16; ++t)
-                    m = min(m, el_of(g0 + t));
-                ((TC *)d.EL)[i] = (TC)m;
-                continue;
+            const long g = i ^ (i >> 1);
+            F acc = 0;
+            for (int r = 0; r < L; ++r) {
+                if (!((g >> r) & 1))
+                    continue;
+                acc += W[(B + r) * n + (B + r)];
+                for (int r2 = r + 1; r2 < L; ++r2)
+                    if ((g >> r2) & 1)
+                        acc += W[(B + r) * n + (B + r2)];
             }
-            const F acc = el_of(i);
+            if constexpr (Tr<T>::kGrouped) {
+                // after E_L, its minimum over each group of 16 walk steps, as stored: 16 consecutive
+                // entries are 16 aligned lanes (rounding to TC is monotonic)
+                if (L >= 4) {
+                    const unsigned half = 0xffffu << (threadIdx.x & 16);
+                    F m = acc;
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1)
+                        m = min(m, __shfl_xor_sync(half, m, o));
+                    if ((i & 15) == 0) {
+                        if constexpr (kPacked)
+                            ((TP *)d.EL)[NL + i / 16] = (TP)m - kLaneBias;
+                        else
+                            ((TC *)d.EL)[NL + i / 16] = (TC)m;
+                    }
+                }
+            }
             if constexpr (kPacked) {
                 if (d.el_fused)  // E_L - elmin in both halves, added to the packed minima of a step
                     ((uint32_t *)d.EL)[i] = (uint32_t)((TP)acc - d.elmin) * 0x10001u;
@@ -604,6 +610,12 @@ __device__ __forceinline__ TC add_min_interleaved(TC (&E)[S], const TC (&M)[S], 
     return tree_min<TC, 3, NL>(l1);
 }
 
+}  // namespace qubo
+
+#include "scan_grouped.cuh"
+
+namespace qubo {
+
 // ---- one work unit: all 2^(B+L) states with fixed bits x_f = unit --------------------------------
 // ADDM >= 4 issues some or all FP32 column adds as paired f32x2 operations (two columns per
 // instruction; 4: all pairs, 5: every second, 6: every fourth, 7: three in four); other modes
@@ -679,54 +691,6 @@ __device__ __forceinline__ void scan_unit(const ScanArgs &a, const Inst &d, int 
             for (int e = 0; e < V; ++e)
                 Mr[r][g * V + e] = (TC)((F)mv[e] + wr);
         }
-    }
-
-    // Step form 2 (integers in FP32 lanes): the walk runs in groups of 16 states, and a group
-    // skips the min tree when no column of it can reach the threshold.  At a group's first state
-    // the exact column minimum m of each thread is taken; a register-row step adds +-M_r[q] to
-    // column q, so over the group's next 15 steps (rows 0-3, the same pattern in every group but
-    // for the sign of row 3, which alternates) the minimum never falls below m + D, D the
-    // smallest running sum of the steps' smallest column moves (min_q M_r[q] on an add,
-    // -max_q M_r[q] on a subtract), computed once per unit in int32 and rounded down.  With
-    // min E_L over the group's states (a table), m + D > uc - min E_L in every lane proves that
-    // the group holds no candidate, and it runs its adds alone.  m + D is summed rounding down;
-    // with integers in FP32 lanes uc - min E_L is exact (|uc|, |E_L| and their difference stay
-    // below 2^24).  FP32 columns take 16 ulp of beta (geps) off the left side, more than the
-    // rounding of the group's 15 adds and of the E_L add the interleaved form compares, and round
-    // uc - min E_L up, so a group is skipped only when the interleaved form records nothing in it.
-    constexpr bool BOUND = ILV == 2 && Tr<T>::kGrouped;
-    static_assert(!BOUND || (RC >= 4 && MINM == 3), "the grouped form needs register rows 0-3 and 3-input mins");
-    // D per parity of the group index, rounded down to FP32 (summed exactly in int64 for integer
-    // columns, in FP64 for FP32 columns, whose table rows are FP32 values)
-    using DD = std::conditional_t<Tr<T>::kFloat, double, int64_t>;
-    float Dgrp[2] = {0, 0};
-    if constexpr (BOUND) {
-        DD dpos[4], dneg[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            TC lo = Mr[r][0], hi = Mr[r][0];
-#pragma unroll
-            for (int q = 1; q < S; ++q) {
-                lo = emin(lo, Mr[r][q]);
-                hi = hi > Mr[r][q] ? hi : Mr[r][q];
-            }
-            dpos[r] = (DD)lo;
-            dneg[r] = -(DD)hi;
-        }
-        static_for<2>([&](auto pc) {
-            constexpr int par = decltype(pc)::value;
-            DD cum = 0, lo = 0;
-            static_for<15>([&](auto tc) {
-                constexpr int t = decltype(tc)::value + 1, kk = ctzc(t);
-                constexpr bool neg = kk == 3 ? par != 0 : ((t >> (kk + 1)) & 1) != 0;
-                cum += neg ? dneg[kk] : dpos[kk];
-                lo = min(lo, cum);
-            });
-            if constexpr (Tr<T>::kFloat)
-                Dgrp[par] = __double2float_rd(lo);
-            else
-                Dgrp[par] = __ll2float_rd(lo);
-        });
     }
 
     // Threshold: a state is recorded when its energy is <= Treg (+ margin).
@@ -820,7 +784,6 @@ __device__ __forceinline__ void scan_unit(const ScanArgs &a, const Inst &d, int 
 
     if (!QUBO_DCHECK(L >= RC + 1 && L <= kMaxWalkBits && nblk * BODY == (1 << L), st, 3))
         return;
-    const TC *ELg = ELp + (1 << L);  // step form 2: min E_L over each group of 16 states
     for (int blk = 0; blk < nblk; ++blk) {
         const int i0 = blk * BODY;
         if constexpr (Tr<T>::kFloat) {
@@ -834,55 +797,6 @@ __device__ __forceinline__ void scan_unit(const ScanArgs &a, const Inst &d, int 
         // moves the threshold) of (minimum over the columns + E_L of the step); a column can be
         // at or below the threshold exactly when its half's minimum is at or below uc.
         TC acc_lo, acc_hi, mprev;
-        if constexpr (BOUND) {
-            constexpr int NG = BODY / 16;
-            TC elg[NG];
-#pragma unroll
-            for (int g = 0; g < NG; ++g)
-                elg[g] = ELg[(i0 >> 4) + g];
-            static_for<NG>([&](auto gc) {
-                constexpr int g = decltype(gc)::value, p0 = 16 * g;
-                if constexpr (g > 0) {  // the step into the group's first state
-                    constexpr int kk = ctzc(p0);
-                    if constexpr (kk < RC) {
-                        add_row<TC, S, ADDM, ((p0 >> (kk + 1)) & 1) != 0>(E, Mr[kk]);
-                    } else {
-                        Pmid = P;
-                        high_flip(RC, (blk & 1) ? -1 : 1);
-                    }
-                }
-                const TC m0 = tree_min<TC, MINM, S>(E);
-                bool clear;
-                if constexpr (Tr<T>::kFloat)  // less the rounding of the group's adds and E_L add
-                    clear = __fadd_rd(__fadd_rd(m0, Dgrp[g & 1]), -d.geps) > __fsub_ru(uc, elg[g]);
-                else
-                    clear = __fadd_rd(m0, Dgrp[g & 1]) > uc - elg[g];
-                const bool skip = __all_sync(kFull, clear);
-                if (__builtin_expect(skip, 1)) {
-                    static_for<15>([&](auto tc) {
-                        constexpr int t = decltype(tc)::value + 1, p = 16 * decltype(gc)::value + t, kk = ctzc(t);
-                        add_row<TC, S, ADDM, ((p >> (kk + 1)) & 1) != 0>(E, Mr[kk]);
-                    });
-                } else {
-                    // the group's states as in the interleaved form: column minima + E_L, running
-                    // minimum compared with the threshold at the group's end
-                    TC ev[V], rm;
-                    static_for<16>([&](auto tc) {
-                        constexpr int t = decltype(tc)::value, p = 16 * decltype(gc)::value + t, kk = t > 0 ? ctzc(t) : 0;
-                        TC mc;
-                        if constexpr (t == 0)
-                            mc = m0;
-                        else
-                            mc = add_min_interleaved<TC, S, ADDM, ((p >> (kk + 1)) & 1) != 0>(E, Mr[kk], (TC)a.zero);
-                        if constexpr (t % V == 0)
-                            vload<TC>(ELp + i0 + p, ev);
-                        const TC mp = mc + ev[t % V];
-                        rm = t == 0 ? mp : emin(rm, mp);
-                    });
-                    hit = hit || rm <= uc;
-                }
-            });
-        } else {
         // Fast path: per step one add per column, a min over the columns, one add of the step's
         // E_L and half a 3-input min into the running minimum; one compare per half body.
         static_for<BODY>([&](auto pc) {
@@ -921,7 +835,6 @@ __device__ __forceinline__ void scan_unit(const ScanArgs &a, const Inst &d, int 
                 hit = acc_lo <= uc;  // before the row-RC flip moves uc
         });
         hit = hit || acc_hi <= uc;
-        }
         if (hit) {
             // Slow path (rare): rebuild every step of this body from the body-end registers and
             // record each column at or below the threshold.  Step p differs from the last step
@@ -1235,7 +1148,7 @@ __device__ __forceinline__ void scan_unit_packed(const ScanArgs &a, const Inst &
 
 
     };
-    if constexpr (ILV == 2) {
+    if constexpr (ILV == 3) {
         // fused-only kernel: the host runs it only on plans whose E_L is fused
         if (QUBO_DCHECK(d.el_fused, st, 8))
             walk(std::true_type{});
@@ -1316,19 +1229,27 @@ __global__ void __launch_bounds__(kScanThreads, MINB) scan_kernel(const ScanArgs
 {
     using TC = typename Tr<T>::TC;
     using TP = typename Tr<T>::TP;
-    constexpr int kAncWarps = Tr<T>::kFloat ? kScanThreads / 32 : 1;  // float scans: re-anchoring base
-    __shared__ TC stage_all[kScanThreads / 32][S * 32];
-    __shared__ __align__(16) TC anc_all[kAncWarps][Tr<T>::kFloat ? S * 32 : 1];
-    __shared__ TP wsm_all[kScanThreads / 32][kMaxWalkBits];
+    // per warp, at constant offsets from one pointer: the hit handlers' staging, the grouped form's
+    // negative row parts, the float scans' re-anchoring base, the walked rows' couplings
+    constexpr int kCols = S * 32;
+    constexpr int kNeg = kCols, kAnc = kNeg + (ILV == 2 ? kCols : 0), kWarpWords = kAnc + (Tr<T>::kFloat ? kCols : 0);
+    struct WarpShared {
+        TC cols[kWarpWords];
+        TP wsm[kMaxWalkBits];
+    };
+    __shared__ __align__(16) WarpShared sh_all[kScanThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    TC *stage = stage_all[warp];
-    TC *anc = anc_all[Tr<T>::kFloat ? warp : 0];
-    TP *wsm = wsm_all[warp];
+    TC *stage = sh_all[warp].cols, *neg = stage + kNeg, *anc = stage + kAnc;
+    TP *wsm = sh_all[warp].wsm;
     TP Treg = (TP)0;
     // units take 0.1-30 ms here: one per claim keeps the end of a launch balanced
     persistent_units<T, 1>(a, lane, Treg, [&](const Inst &d, int inst, uint64_t unit) {
-        if constexpr (Tr<T>::kPack == 2)
+        if constexpr (Tr<T>::kPack == 2 && ILV == 2)
+            scan_unit_packed_grouped<S, RC, RC == 5 ? kLongBody : 1, K1>(a, d, inst, unit, Treg, lane, stage, wsm, neg);
+        else if constexpr (Tr<T>::kPack == 2)
             scan_unit_packed<S, RC, K1, ADDM, MINM, ILV>(a, d, inst, unit, Treg, lane, stage, wsm);
+        else if constexpr (ILV == 2)
+            scan_unit_grouped<T, S, RC, RC == 5 ? kLongBody : 1, K1, ADDM>(a, d, inst, unit, Treg, lane, stage, wsm, anc, neg);
         else
             scan_unit<T, S, RC, K1, ADDM, MINM, ILV>(a, d, inst, unit, Treg, lane, stage, wsm, anc);
     });

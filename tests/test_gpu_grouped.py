@@ -1,0 +1,108 @@
+"""The grouped step form of the int32 and packed 16-bit scans against the CPU oracle, at the sizes
+where it can go wrong: the shortest walks (one group per body, one body per unit), walks across
+several memory rows, entries at the limits its arithmetic admits (packed columns up to the cap of
+its adds, int32 energies near 2^30), and instances whose groups mostly or always reach the threshold
+(small integers, ties everywhere, a wide energy window)."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2607_04857_gb300 import workloads as wl
+from plan_checks import column_range
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def q():
+    import paper_2607_04857_gb300 as q
+
+    q.load_library()
+    return q
+
+
+@pytest.fixture(autouse=True)
+def dense(monkeypatch):
+    monkeypatch.setenv("QUBO_NO_I32Z", "1")
+
+
+def check(r, o):
+    assert r.min == o.min and r.n_ties == o.n_ties
+    assert np.array_equal(r.ties, o.ties) and np.array_equal(r.topk, o.topk) and np.array_equal(r.topk_E, o.topk_E)
+
+
+@pytest.mark.parametrize("acc,variant", [("i16p", 20), ("i16p", 21), ("i32", 20), ("i32", 21)])
+@pytest.mark.parametrize("walk", [5, 6, 7, 11, 14])
+def test_walks(q, acc, variant, walk, monkeypatch):
+    if walk == 5 and variant == 20:
+        pytest.skip("five register rows need six walked bits")
+    monkeypatch.setenv("QUBO_SCAN_VARIANT", str(variant))
+    Q = wl.upper_int(26, -90, 90, seed=walk + variant)
+    o = oracle.solve(Q, topk=12)
+    r = q.solve(Q, topk=12, walk_bits=walk, int32=acc == "i32")
+    assert (r.info["acc"], r.info["grouped"], r.info["walk_bits"]) == (acc, 1, walk), r.info
+    check(r, o)
+    check(q.solve(Q, walk_bits=walk, int32=acc == "i32"), oracle.solve(Q))
+
+
+@pytest.mark.parametrize("scale", [1.0, 1.0005, 1.01, 1.3])
+def test_packed_limits(q, scale):
+    """Columns scaled up to 32767: the grouped form runs while none reaches 32767 and the rows' moves
+    fit 16 bits, its interleaved twin beyond (both exact), other accumulators past 16 bits."""
+    Q = wl.upper_int(24, -1000, 1000, seed=31)
+    hi = max(column_range(Q, 10, 6, 5)[1], -column_range(Q, 10, 6, 5)[0])
+    Q = (Q * (32766.0 / hi * scale)).astype(np.int32)
+    r = q.solve(Q, topk=8, walk_bits=6)
+    lo, hi = column_range(Q, 10, 6, 5)
+    assert (r.info["acc"] == "i16p") == (lo >= -32768 and hi <= 32767)
+    if r.info["grouped"] and r.info["acc"] == "i16p":
+        assert hi < 32767
+    check(r, oracle.solve(Q, topk=8))
+
+
+@pytest.mark.parametrize("sign", [-1, 0, 1])
+def test_int32_limits(q, sign):
+    """Energies up to the int32 bound (sum of |U| just below 2^30), of both signs and of one."""
+    Q = wl.upper_int(23, 1, 1 << 20, seed=40)
+    Q = Q * np.where((sign > 0) | ((sign == 0) & (np.arange(23 * 23).reshape(23, 23) % 2 == 1)), 1, -1)
+    Q = (Q.astype(np.float64) * ((2.0**30 - 600) / np.abs(np.triu(Q)).astype(np.float64).sum())).astype(np.int32)
+    assert np.abs(Q.astype(np.int64)).sum() < 1 << 30
+    r = q.solve(Q, topk=8)
+    assert r.info["acc"] == "i32" and r.info["grouped"] == 1, r.info
+    check(r, oracle.solve(Q, topk=8))
+
+
+@pytest.mark.parametrize("acc", ["i16p", "i32"])
+def test_every_group_reaches_the_threshold(q, acc):
+    """Ties in every group (10 diagonal entries of -1, the other variables free), and +-1 couplings."""
+    Q = np.zeros((24, 24), dtype=np.int32)
+    Q[np.arange(10), np.arange(10)] = -1
+    kw = dict(int32=acc == "i32", walk_bits=9)
+    check(q.solve(Q, states_cap=1 << 14, **kw), oracle.solve(Q, cap=1 << 14))
+    Q = wl.upper_int(24, -1, 1, seed=2)
+    r = q.solve(Q, topk=40, states_cap=4096, **kw)
+    assert r.info["acc"] == acc and r.info["grouped"] == 1
+    check(r, oracle.solve(Q, topk=40, cap=4096))
+
+
+def test_window_and_sub_cubes(q):
+    Q = wl.upper_int(30, -120, 120, seed=5)
+    o = oracle.solve(Q, topk=4096, cap=1, fix_bits=6, fix_value=11)
+    width = int(o.topk_E[1500] - o.min)
+    sel = o.topk_E <= o.min + width
+    assert not sel.all()
+    cnt, codes, E, info = q.solve_window(Q, width, fix_bits=6, fix_value=11)
+    assert info["acc"] == "i16p" and cnt == int(sel.sum())
+    assert np.array_equal(codes, o.topk[sel]) and np.array_equal(E, o.topk_E[sel])
+    for v in (0, 63):
+        check(q.solve(Q, topk=5, fix_bits=6, fix_value=v), oracle.solve(Q, topk=5, fix_bits=6, fix_value=v))
+
+
+@pytest.mark.parametrize("count", [1, 3, 40])
+def test_small_batches(q, count):
+    """A small batch's walk is shortened to occupy the GPU; sizes from direct evaluation to 24."""
+    insts = [wl.upper_int(int(n), -100, 100, seed=int(n), dtype=np.int16) for n in np.linspace(24, 11, count)]
+    for Q, r in zip(insts, q.solve_batched(insts, topk=3, states_cap=16)):
+        check(r, oracle.solve(Q.astype(np.int32), topk=3, cap=16))

@@ -90,3 +90,22 @@ def test_group_bound_is_tight_for_one_column():
         neg = (t >> (kk + 1)) & 1  # group 0: the sign of row 3 follows bit 4 of the position (0)
         walk.append(walk[-1] + (-1 if neg else 1) * (M[kk, 0] + w[kk]))
     assert group_bound(M, w, 0) == min(walk)
+
+
+@pytest.mark.parametrize("seed", range(3))
+def test_exact_group_minimum(seed):
+    """The second test's bound: a column's minimum over a group is its value with rows 0-3 clear plus
+    the negative parts of the four rows (rows 0-2 are clear and row 3 follows the group's parity at
+    the group's first state)."""
+    rng = np.random.default_rng(seed)
+    rows, start = rng.integers(-50, 51, size=(4, 8)), rng.integers(-300, 300, size=8)
+    for par in (0, 1):
+        base = start  # rows 0-3 clear
+        first = base + par * rows[3]
+        col, least = first.copy(), first.copy()
+        for t in range(1, 16):
+            kk = (t & -t).bit_length() - 1
+            neg = bool(par) if kk == 3 else bool((t >> (kk + 1)) & 1)
+            col = col + (-1 if neg else 1) * rows[kk]
+            least = np.minimum(least, col)
+        assert np.array_equal(least, first - par * rows[3] + np.minimum(rows, 0).sum(axis=0))
