@@ -96,6 +96,9 @@ static_assert(kMad * kMadInverse == 1u, "the inverse of kMad modulo 2^32");
 constexpr int kScanThreads = 128;
 // Longest Gray walk inside one work unit (also the FP32 re-anchoring period).
 constexpr int kMaxWalkBits = 16;
+// States of one work item of an instance evaluated directly (log2).
+constexpr int kSmallChunkLog2 = 10;
+constexpr uint64_t small_items(uint64_t states) { return states >> kSmallChunkLog2 ? states >> kSmallChunkLog2 : 1; }
 // Batched instances carry their index in the top bits of a candidate key.
 constexpr int kInstShift = 40;
 constexpr int kMaxBatchedN = 40;

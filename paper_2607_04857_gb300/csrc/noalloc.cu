@@ -243,7 +243,7 @@ extern "C" int qubo_solve_noalloc(const void *Q_host, int n, qubo_dtype dtype, i
     is.thr = (unsigned long long)(uint32_t)(int32_t)descent_bound(U, n);
     is.gmin = (unsigned long long)(uint32_t)INT32_MAX;
     std::memcpy(hdr + lo.state, &is, sizeof(is));
-    const uint64_t items[2] = {0, small ? 1ull : (1ull << k)};
+    const uint64_t items[2] = {0, small ? small_items(1ull << n) : (1ull << k)};
     std::memcpy(hdr + lo.items, items, sizeof(items));
     int32_t *W = (int32_t *)(hdr + lo.W);
     for (int a = 0; a < n; ++a)

@@ -187,7 +187,7 @@ int plan(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bi
         h.sub_base = fix_bits ? (fix_value << free_bits) : 0;
         h.sub_count = h.states;
         h.units = 0;
-        h.items = 1;
+        h.items = small_items(h.states);
         return QUBO_OK;
     }
     h.small = 0;

@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) zscan_one_kernel(const ScanAr
             }
             const Inst d = a.inst[inst];
             if (d.small) {
-                small_unit<T>(a, d, inst, lane);  // counts its own states
+                small_unit<T>(a, d, inst, item - a.item_base[inst], lane);  // counts its own states
                 ++item;
                 continue;
             }

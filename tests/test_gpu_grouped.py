@@ -106,3 +106,26 @@ def test_small_batches(q, count):
     insts = [wl.upper_int(int(n), -100, 100, seed=int(n), dtype=np.int16) for n in np.linspace(24, 11, count)]
     for Q, r in zip(insts, q.solve_batched(insts, topk=3, states_cap=16)):
         check(r, oracle.solve(Q.astype(np.int32), topk=3, cap=16))
+
+
+# --- direct evaluation (sub-cubes too small to split) ------------------------------------------
+
+@pytest.mark.parametrize("free", [0, 1, 4, 5, 6, 9, 10, 11, 12, 13])
+def test_direct_evaluation(q, free):
+    """Items of 2^10 states: fewer states than lanes, one partial item, several; variables above the
+    sub-cube fixed to patterns with both values, up to variable 63; every accumulator."""
+    for n, fix in ((free, 0), (40, 0x15555), (64, (1 << 40) + 12345)):
+        if n < max(free, 1):
+            continue
+        fb = n - free
+        fv = fix & ((1 << fb) - 1)
+        K = min(1 << free, 20)
+        Q = wl.upper_int(n, -1000, 1000, seed=free + n)
+        wide = wl.upper_int(n, -(1 << 30), 1 << 30, seed=free + n)
+        for M in (Q, wide, Q.astype(np.int16)):
+            check(q.solve(M, topk=K, fix_bits=fb, fix_value=fv),
+                  oracle.solve(M.astype(np.int32), topk=K, fix_bits=fb, fix_value=fv))
+        F = wl.sk_float32(n, seed=free + n)
+        for kw in ({}, {"plain": True}):
+            r, o = q.solve(F, topk=K, fix_bits=fb, fix_value=fv, **kw), oracle.solve(F, topk=K, fix_bits=fb, fix_value=fv)
+            assert r.min == o.min and np.array_equal(r.topk, o.topk) and np.array_equal(r.ties, o.ties)
