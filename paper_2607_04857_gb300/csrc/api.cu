@@ -474,6 +474,8 @@ int job_layout(Job &j)
     o = align_up(o + sizeof(Inst) * ni, 256);
     j.off_state = o;
     o = align_up(o + sizeof(InstState) * ni, 256);
+    j.off_ctr = o;  // queue and record counters, zero at every run's start as the state is reset
+    o = align_up(o + 16 * 8, 256);
     j.off_items = o;
     o = align_up(o + sizeof(uint64_t) * (ni + 1), 256);
     j.off_W.resize(ni);
@@ -528,11 +530,9 @@ int job_layout(Job &j)
     j.off_topke = o;
     o = align_up(o + 8 * (size_t)j.K * ni, 256);
     j.off_starts = o;
-    o = align_up(o + 16 * (size_t)ni, 256);
-    j.off_ctr = o;
-    o = align_up(o + 16 * 8, 256);
+    o = align_up(o + 16 * (size_t)ni + 8, 256);
     j.arena_bytes = o;
-    d = sizeof(ResOut) * ni + sizeof(InstState) * ni + 8 * j.cap * ni + 16 * (size_t)j.K * ni + 16 * 8 + 4096;
+    d = 64 + sizeof(ResOut) * ni + sizeof(InstState) * ni + 8 * j.cap * ni + 16 * (size_t)j.K * ni + 4096;
     j.down_bytes = d;
     return QUBO_OK;
 }
@@ -558,6 +558,7 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
         total += j.insts[i]->items;
     }
     items[ni] = total;
+    std::memset(up + j.off_ctr, 0, 16 * 8);
     // descriptors, initial state and coupling matrices; instances write disjoint regions
     auto stage_one = [&](int i) {
         HostInst &h = *j.insts[i];
@@ -645,7 +646,8 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
             stage_one(i);
     });
     j.total_items = total;
-    j.rec_cap = std::min(ws.rec_cap, record_capacity());
+    // a batch's records are moved to per-instance segments in the buffer's upper half
+    j.rec_cap = std::min(ni > 1 ? ws.rec_cap / 2 : ws.rec_cap, record_capacity());
     int bps = scan_blocks_per_sm(j.acc, j.K <= 1, j.variant);
     if (bps < 1)
         bps = 1;
@@ -666,12 +668,11 @@ int job_enqueue_scan(Workspace &ws, Job &j, const void *state_init = nullptr)
     char *dev = (char *)ws.d_arena;
     cudaStream_t s = j.stream;
     if (state_init) {
-        CK(cudaMemcpyAsync(dev + j.off_state, state_init, sizeof(InstState) * ni, cudaMemcpyDeviceToDevice, s));
+        CK(cudaMemcpyAsync(dev + j.off_state, state_init, j.off_items - j.off_state, cudaMemcpyDeviceToDevice, s));
     } else {
         CK(cudaMemcpyAsync(dev, up, j.up_bytes, cudaMemcpyHostToDevice, s));
         j.h2d += j.up_bytes;
     }
-    CK(cudaMemsetAsync(dev + j.off_ctr, 0, 16 * 8, s));
     CK(record_event(ws.ev[0], s));
     CK(launch_tables(j.acc, (const Inst *)(dev + j.off_inst), ni, j.max_entries, s));
     CK(record_event(ws.ev[3], s));
@@ -698,20 +699,22 @@ int job_enqueue_scan(Workspace &ws, Job &j, const void *state_init = nullptr)
     return QUBO_OK;
 }
 
-// Stage, upload and launch tables + scan.  Does not wait.
+int job_enqueue_finish(Workspace &ws, Job &j);
+
+// Stage, upload and launch tables, scan and the short-list finalization.  Does not wait.
 int job_launch(Workspace &ws, Job &j)
 {
     int st;
     if ((st = job_stage(ws, j)))
         return st;
     *ws.h_abort = g_abort_all.load() ? 1 : 0;
-    if ((st = job_enqueue_scan(ws, j)))
+    if ((st = job_enqueue_scan(ws, j)) || (st = job_enqueue_finish(ws, j)))
         return st;
     j.t_start = now_s();
     return QUBO_OK;
 }
 
-// Wait for `ev` (the scan's end), honouring the time limit and qubo_abort.
+// Wait for `ev` (the run's end), honouring the time limit and qubo_abort.
 int job_wait(Workspace &ws, Job &j, cudaEvent_t ev)
 {
     for (;;) {
@@ -736,6 +739,7 @@ int job_wait(Workspace &ws, Job &j, cudaEvent_t ev)
 
 // Host-side view of the download staging buffer.
 struct Down {
+    unsigned long long *hdr;
     ResOut *res;
     InstState *sts;
     uint64_t *ties, *tk;
@@ -747,7 +751,8 @@ Down down_view(Workspace &ws, const Job &j)
     const int ni = (int)j.insts.size();
     char *down = (char *)ws.h_down;
     Down d;
-    size_t o = 0;
+    size_t o = 64;
+    d.hdr = (unsigned long long *)down;
     d.res = (ResOut *)(down + o);
     o += sizeof(ResOut) * ni;
     d.sts = (InstState *)(down + o);
@@ -846,29 +851,61 @@ Part part_from(const Down &d, const Job &j, int i)
     return p;
 }
 
-// Wait for the scan, finalize with the exact record count, download and unpack.
-int job_finish(Workspace &ws, Job &j, std::vector<Part> &parts, double *gpu_seconds)
+// Enqueue the short-list finalization (launch_finish) behind the scan: no count is read back, and the
+// results land in the staging buffer.
+int job_enqueue_finish(Workspace &ws, Job &j)
 {
+    const int ni = (int)j.insts.size();
     char *dev = (char *)ws.d_arena;
-    int st;
-    if ((st = job_wait(ws, j, ws.ev[1])))
-        return st;
-    unsigned long long nrec = 0;
-    CK(cudaMemcpy(&nrec, dev + j.off_ctr + 8, 8, cudaMemcpyDeviceToHost));
+    const Down d = down_view(ws, j);
+    const FinishOut o{d.hdr, d.res, d.sts, d.ties, d.tk, d.tke};
+    CK(launch_finish((const Inst *)(dev + j.off_inst), (InstState *)(dev + j.off_state), ws.d_rec,
+                     ws.d_rec + ws.rec_cap / 2, (const unsigned long long *)(dev + j.off_ctr) + 1, j.rec_cap, ni,
+                     acc_float(j.acc), j.window >= 0.0, j.K, j.cap, (unsigned long long *)(dev + j.off_starts), o,
+                     j.stream, &j.launches));
+    CK(record_event(ws.ev[2], j.stream));
+    return QUBO_OK;
+}
+
+// After the run has finished: when an instance's record list was too long for the short-list
+// finalization, sort and extract all of them by the general path, and wait for it.
+int job_long_lists(Workspace &ws, Job &j)
+{
+    const int ni = (int)j.insts.size();
+    const Down d = down_view(ws, j);
+    const unsigned long long cnt = std::min<unsigned long long>(d.hdr[0], j.rec_cap);
+    bool longer = false;
+    for (int i = 0; i < ni; ++i) {
+        longer = longer || d.res[i].has == 2;
+        j.d2h += sizeof(ResOut) + sizeof(InstState) + 8 * d.res[i].n_written + 16 * (size_t)d.res[i].nk;
+    }
     j.d2h += 8;
-    const unsigned long long cnt = std::min(nrec, j.rec_cap);
+    if (!longer)
+        return QUBO_OK;
     unsigned long long P = 1;
     while (P < cnt)
         P <<= 1;
+    int st;
     if ((st = job_enqueue_finalize(ws, j, cnt, P)))
         return st;
+    CK(cudaStreamSynchronize(j.stream));
+    return QUBO_OK;
+}
+
+// Wait for the run and unpack its results.
+int job_finish(Workspace &ws, Job &j, std::vector<Part> &parts, double *gpu_seconds)
+{
+    int st;
+    if ((st = job_wait(ws, j, ws.ev[2])) || (st = job_long_lists(ws, j)))
+        return st;
+    const unsigned long long cnt = std::min<unsigned long long>(down_view(ws, j).hdr[0], j.rec_cap);
     std::vector<Rec> sorted;
     if (j.window >= 0.0 && cnt) {
         sorted.resize(cnt);
         CK(cudaMemcpyAsync(sorted.data(), ws.d_rec, sizeof(Rec) * cnt, cudaMemcpyDeviceToHost, j.stream));
+        CK(cudaStreamSynchronize(j.stream));
         j.d2h += sizeof(Rec) * cnt;
     }
-    CK(cudaStreamSynchronize(j.stream));
     job_unpack(ws, j, parts, gpu_seconds);
     for (size_t i = 0; i < parts.size(); ++i)
         if (parts[i].dbg) {
@@ -1489,6 +1526,7 @@ struct qubo_batch {
     size_t cap = 0;
     bool is_float = false;
     size_t off_state_init = 0;
+    int graph_launches = 0;   // kernels of one replay
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap_stream = nullptr;
@@ -2061,12 +2099,12 @@ int qubo_batch_create(const void *Q_packed, const int *n, const size_t *offsets,
     j.margin = kDefaultMargin;
     j.variant = b->hs[0].variant;
     // the initial per-instance state lives after the job's arena and is copied in at every run
-    const size_t state_bytes = sizeof(InstState) * (size_t)count;
-    if ((st = job_stage(b->ws, j, state_bytes + 256)))
+    // (with the counters behind it)
+    if ((st = job_stage(b->ws, j, align_up(sizeof(InstState) * (size_t)count, 256) + 512)))
         return st;
-    // A graph sorts with a fixed network sized by the buffer; batches produce few candidates per
-    // instance, so a smaller buffer keeps the replay short (an instance that overflows it is
-    // solved again on its own at fetch time).
+    const size_t state_bytes = j.off_items - j.off_state;
+    // Batches produce few candidates per instance (an instance that overflows the buffer is solved again
+    // on its own at fetch time).
     j.rec_cap = std::min<unsigned long long>(j.rec_cap, kBatchGraphRecords);
     b->off_state_init = align_up(j.arena_bytes, 256);
     char *dev_arena = (char *)b->ws.d_arena;
@@ -2074,18 +2112,16 @@ int qubo_batch_create(const void *Q_packed, const int *n, const size_t *offsets,
     CK(cudaMemcpy(dev_arena + b->off_state_init, (char *)b->ws.h_up + j.off_state, state_bytes,
                   cudaMemcpyHostToDevice));
     j.h2d += j.up_bytes + state_bytes;
-    // capture tables -> scan -> (rescore) -> sort -> extract -> download as one graph
+    // capture tables -> scan -> finalization into the staging buffer as one graph
     if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         return QUBO_ERR_CUDA;
     }
     j.stream = b->cap_stream;
-    unsigned long long P = 1;
-    while (P < j.rec_cap)
-        P <<= 1;
     CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
     int st1 = job_enqueue_scan(b->ws, j, dev_arena + b->off_state_init);
-    int st2 = st1 ? st1 : job_enqueue_finalize(b->ws, j, j.rec_cap, P);
+    int st2 = st1 ? st1 : job_enqueue_finish(b->ws, j);
+    b->graph_launches = j.launches;
     const cudaError_t ce = cudaStreamEndCapture(b->cap_stream, &b->graph);
     if (st1 || st2 || ce != cudaSuccess) {
         cudaGetLastError();
@@ -2142,21 +2178,9 @@ int qubo_batch_fetch(qubo_batch *b, void *out_min, uint64_t *out_states, uint64_
         if (cudaEventElapsedTime(&ms, b->ws.ev[3], b->ws.ev[1]) == cudaSuccess)
             j.scan_seconds = ms * 1e-3;
     }
-    // the graph's launches: the same kernels a direct run makes, with every sort stage present
-    {
-        const bool is_float = acc_float(j.acc);
-        unsigned long long P = 1;
-        while (P < j.rec_cap)
-            P <<= 1;
-        int nl = 2 + (is_float ? 1 : 0) + 2 + (P >= 2 ? 2 : 0);
-        for (unsigned long long k = 4096; k <= P; k <<= 1) {
-            for (unsigned long long jj = k >> 1; jj >= 2048; jj >>= 1)
-                ++nl;
-            ++nl;
-        }
-        j.launches = nl;
-    }
-    j.d2h = sizeof(ResOut) * b->count + sizeof(InstState) * b->count + 8 * j.cap * b->count + 16 * (size_t)j.K * b->count;
+    j.launches = b->graph_launches;
+    if ((st = job_long_lists(b->ws, j)))
+        return st;
     if (j.aborted)
         return QUBO_ERR_TIMEOUT;
     const Down d = down_view(b->ws, j);

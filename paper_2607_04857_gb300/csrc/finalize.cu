@@ -292,7 +292,211 @@ __global__ void extract_kernel(const Rec *rec, bool batched, int n_inst, int top
     }
 }
 
+// ---- short record lists: one block per instance sorts, extracts and hands over ------------------
+// The records of an instance are few (tens to hundreds), and the general path above costs them a
+// host round trip for their count, a sort network of full length when captured, and a copy per result
+// array.  finish_kernel reads the count on the device, sorts up to kChunk records in shared memory
+// and writes the results straight to the host's pinned staging buffer; a longer list is left to
+// the general path (FinishOut::hdr, ResOut::has = 2).  A batch's records, interleaved in the buffer,
+// are first moved to one segment per instance.  Latency-bound throughout.
+
+// Exclusive sums of the stored records per instance (one block).
+__global__ void __launch_bounds__(1024) segment_kernel(const InstState *state, int n_inst, unsigned long long *starts,
+                                                       unsigned long long *cursor)
+{
+    __shared__ unsigned long long warp_sums[32], carry;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0)
+        carry = 0;
+    __syncthreads();
+    for (int base = 0; base < n_inst; base += 1024) {
+        const int i = base + (int)threadIdx.x;
+        const unsigned long long c = i < n_inst ? state[i].nrec - state[i].dropped : 0ull;
+        unsigned long long sum = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(kFullMask, sum, o);
+            if (lane >= o)
+                sum += v;
+        }
+        if (lane == 31)
+            warp_sums[warp] = sum;
+        __syncthreads();
+        if (warp == 0) {
+            unsigned long long w = warp_sums[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long v = __shfl_up_sync(kFullMask, w, o);
+                if (lane >= o)
+                    w += v;
+            }
+            warp_sums[lane] = w;
+        }
+        __syncthreads();
+        const unsigned long long excl = carry + (warp ? warp_sums[warp - 1] : 0ull) + sum - c;
+        if (i < n_inst) {
+            starts[i] = excl;
+            cursor[i] = excl;
+        }
+        __syncthreads();
+        if (threadIdx.x == 1023)
+            carry = excl + c;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0)
+        starts[n_inst] = carry;
+}
+
+// Move every record to its instance's segment; float records are rescored on the way.
+template <bool FL>
+__global__ void scatter_kernel(const Inst *insts, InstState *state, const Rec *rec, const unsigned long long *d_nrec,
+                               unsigned long long cap, int n_inst, unsigned long long *cursor, Rec *out)
+{
+    const unsigned long long cnt = rec_count(d_nrec, cap);
+    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
+         i += (unsigned long long)gridDim.x * blockDim.x) {
+        Rec r = rec[i];
+        const uint64_t inst = rec_inst(r.key, true);
+        if (inst >= (uint64_t)n_inst)
+            continue;
+        if constexpr (FL) {
+            const double e64 = energy_fp64(insts[inst].U64, insts[inst].n, rec_code(r.key, true));
+            atomicMax(&state[inst].err,
+                      (unsigned long long)__double_as_longlong(fabs(__longlong_as_double(r.e) - e64)));
+            r.e = __double_as_longlong(e64);
+        }
+        const unsigned long long pos = atomicAdd(cursor + inst, 1ull);
+        if (pos < cap)
+            out[pos] = r;
+    }
+}
+
+// Block b: instance b.  Single instance (batched false): all records, rescored here for floats and,
+// with write_back, stored sorted.
+template <bool FL>
+__global__ void __launch_bounds__(512) finish_kernel(const Inst *insts, InstState *state, Rec *rec,
+                                                     const unsigned long long *d_nrec, unsigned long long cap,
+                                                     const unsigned long long *starts, bool batched, bool write_back,
+                                                     int topk, unsigned long long states_cap, FinishOut o)
+{
+    __shared__ Rec sh[kChunk];
+    __shared__ unsigned n_ties, n_near;
+    __shared__ unsigned long long err;
+    const int inst = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    const unsigned long long first = batched ? starts[inst] : 0ull;
+    const unsigned long long count = (batched ? starts[inst + 1] : rec_count(d_nrec, cap)) - first;
+    if (inst == 0 && tid == 0)
+        o.hdr[0] = *d_nrec;
+    ResOut out{};
+    if (count > (unsigned long long)kChunk) {
+        if (tid == 0) {
+            out.has = 2;
+            o.res[inst] = out;
+            o.sts[inst] = state[inst];
+        }
+        return;
+    }
+    const unsigned cnt = (unsigned)count, P = (unsigned)pow2_ceil(count);
+    if (tid == 0) {
+        n_ties = n_near = cnt;
+        err = state[inst].err;
+    }
+    __syncthreads();
+    for (unsigned t = tid; t < P; t += nt) {
+        Rec r;
+        if (t < cnt) {
+            r = rec[first + t];
+            if (FL && !batched) {
+                const double e64 = energy_fp64(insts[inst].U64, insts[inst].n, r.key);
+                atomicMax(&err, (unsigned long long)__double_as_longlong(fabs(__longlong_as_double(r.e) - e64)));
+                r.e = __double_as_longlong(e64);
+            }
+        } else {
+            r.key = ~0ull;
+            r.e = FL ? 0x7ff0000000000000ll : 0x7fffffffffffffffll;
+        }
+        sh[t] = r;
+    }
+    __syncthreads();
+    for (unsigned k = 2; k <= P; k <<= 1)
+        for (unsigned j = k >> 1; j > 0; j >>= 1) {
+            for (unsigned t = tid; t < P; t += nt) {
+                const unsigned l = t ^ j;
+                if (l > t) {
+                    const Rec a = sh[t], b = sh[l];
+                    // within a segment every key has the same instance
+                    if ((t & k) == 0 ? rec_less<FL>(b, a, false) : rec_less<FL>(a, b, false)) {
+                        sh[t] = b;
+                        sh[l] = a;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    const int64_t emin = sh[0].e;
+    const double fmin = __longlong_as_double(emin), near_lim = fmin + 1e-9 * fmax(1.0, fabs(fmin));
+    for (unsigned t = tid; t < cnt; t += nt) {  // the ties and the near-ties are prefixes
+        if (sh[t].e != emin)
+            atomicMin(&n_ties, t);
+        if (FL && !(__longlong_as_double(sh[t].e) <= near_lim))
+            atomicMin(&n_near, t);
+        if (write_back)
+            rec[first + t] = sh[t];
+    }
+    __syncthreads();
+    const unsigned ties = n_ties;
+    const unsigned nw = ties < states_cap ? ties : (unsigned)states_cap, nk = cnt < (unsigned)topk ? cnt : (unsigned)topk;
+    for (unsigned t = tid; t < nw; t += nt)
+        o.ties[(unsigned long long)inst * states_cap + t] = rec_code(sh[t].key, batched);
+    for (unsigned t = tid; t < nk; t += nt) {
+        o.topk[(size_t)inst * topk + t] = rec_code(sh[t].key, batched);
+        o.topke[(size_t)inst * topk + t] = sh[t].e;
+    }
+    if (tid == 0) {
+        if (cnt) {
+            out.min_i = emin;
+            out.min_f = FL ? fmin : (double)emin;
+            out.n_ties = ties;
+            out.n_written = nw;
+            out.n_near = FL ? n_near : ties;
+            out.nk = (int32_t)nk;
+            out.has = 1;
+        }
+        o.res[inst] = out;
+        InstState st = state[inst];
+        st.err = err;
+        o.sts[inst] = st;
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_finish(const Inst *d_inst, InstState *d_state, Rec *rec, Rec *segments,
+                          const unsigned long long *d_nrec, unsigned long long cap, int n_inst, bool is_float,
+                          bool write_back, int topk, unsigned long long states_cap, unsigned long long *d_starts,
+                          const FinishOut &o, cudaStream_t s, int *launches)
+{
+    const bool batched = n_inst > 1;
+    if (batched) {
+        unsigned long long *cursor = d_starts + n_inst + 1;
+        segment_kernel<<<1, 1024, 0, s>>>(d_state, n_inst, d_starts, cursor);
+        const int blocks = n_inst < 65536 ? (n_inst + 15) / 16 : 4096;  // a few records per instance
+        if (is_float)
+            scatter_kernel<true><<<blocks, 256, 0, s>>>(d_inst, d_state, rec, d_nrec, cap, n_inst, cursor, segments);
+        else
+            scatter_kernel<false><<<blocks, 256, 0, s>>>(d_inst, d_state, rec, d_nrec, cap, n_inst, cursor, segments);
+        rec = segments;
+    }
+    const int threads = batched ? 128 : 512;
+    if (is_float)
+        finish_kernel<true><<<n_inst, threads, 0, s>>>(d_inst, d_state, rec, d_nrec, cap, d_starts, batched, write_back,
+                                                       topk, states_cap, o);
+    else
+        finish_kernel<false><<<n_inst, threads, 0, s>>>(d_inst, d_state, rec, d_nrec, cap, d_starts, batched,
+                                                        write_back, topk, states_cap, o);
+    *launches += batched ? 3 : 1;
+    return cudaGetLastError();
+}
 
 cudaError_t launch_rescore(const Inst *d_inst, InstState *d_state, Rec *rec, const unsigned long long *d_nrec,
                            unsigned long long cap, bool batched, unsigned long long max_count, cudaStream_t s)

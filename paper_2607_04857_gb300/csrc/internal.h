@@ -168,7 +168,17 @@ struct ResOut {
     unsigned long long n_written;
     unsigned long long n_near;
     int32_t nk;
-    int32_t has;
+    int32_t has;  // 1: results; 2 (finish_kernel): more records than it sorts, nothing extracted
+};
+
+// Where finish_kernel writes (the host's pinned staging buffer): hdr[0] = candidates offered, then per
+// instance the result, the final state, the tie codes and the K lowest.
+struct FinishOut {
+    unsigned long long *hdr;
+    ResOut *res;
+    InstState *sts;
+    uint64_t *ties, *topk;
+    int64_t *topke;
 };
 
 struct ScanArgs {
@@ -231,6 +241,12 @@ cudaError_t launch_extract(const Inst *d_inst, const Rec *rec, const unsigned lo
                            int n_inst, bool batched, bool is_float, int topk, unsigned long long states_cap,
                            ResOut *res, uint64_t *ties, uint64_t *topk_codes, int64_t *topk_e,
                            unsigned long long *d_starts, cudaStream_t s);
+// Sort and extract record lists of up to 2048 records per instance, results to o; `segments` (cap
+// records) and d_starts (2 n_inst + 1 words) are scratch of a batch.
+cudaError_t launch_finish(const Inst *d_inst, InstState *d_state, Rec *rec, Rec *segments,
+                          const unsigned long long *d_nrec, unsigned long long cap, int n_inst, bool is_float,
+                          bool write_back, int topk, unsigned long long states_cap, unsigned long long *d_starts,
+                          const FinishOut &o, cudaStream_t s, int *launches);
 
 // ---- host state shared by the entry points (api.cu) --------------------------------------------
 // True while qubo_abort() is in force (until qubo_abort_clear()).

@@ -129,3 +129,30 @@ def test_direct_evaluation(q, free):
         for kw in ({}, {"plain": True}):
             r, o = q.solve(F, topk=K, fix_bits=fb, fix_value=fv, **kw), oracle.solve(F, topk=K, fix_bits=fb, fix_value=fv)
             assert r.min == o.min and np.array_equal(r.topk, o.topk) and np.array_equal(r.ties, o.ties)
+
+
+# --- record lists: sorted and extracted on the device, short and long --------------------------
+
+@pytest.mark.parametrize("zeros", [0, 5, 10, 11, 12, 16])
+def test_record_list_lengths(q, zeros):
+    """2^zeros minimisers: lists of one record, up to the short list's 2048 and beyond, alone and in a
+    batch beside short ones (single calls and graph replays), integer and float."""
+    Q = wl.diagonal(18, seed=3, zeros=zeros)
+    o = oracle.solve(Q, topk=30, cap=5000)
+    check(q.solve(Q, topk=30, states_cap=5000), o)
+    few = wl.upper_int(17, -50, 50, seed=9)
+    of = oracle.solve(few, topk=30, cap=5000)
+    b = q.Batch([few, Q, few, Q], topk=30, states_cap=5000)
+    for _ in range(2):
+        b.run()
+        for rs in (q.solve_batched([few, Q, few, Q], topk=30, states_cap=5000), b.fetch()):
+            for r, e in zip(rs, (of, o, of, o)):
+                check(r, e)
+        b.run()
+    b.fetch()
+    b.close()
+    F = Q.astype(np.float32)
+    r = q.solve(F, topk=30, states_cap=5000)
+    assert r.min == o.min and r.n_ties == o.n_ties and np.array_equal(r.ties, o.ties) and np.array_equal(r.topk, o.topk)
+    for r, e in zip(q.solve_batched([few.astype(np.float32), F], topk=30, states_cap=5000), (of, o)):
+        assert r.min == e.min and r.n_ties == e.n_ties and np.array_equal(r.ties, e.ties)
