@@ -463,6 +463,7 @@ struct Job {
     double scan_seconds = 0.0;
     uint64_t total_items = 0;
     double window = -1.0;  // >= 0: energy-window mode (single instance)
+    unsigned long long give_up_records = 0;  // SolveCfg::give_up_records
 };
 
 int job_layout(Job &j)
@@ -648,6 +649,8 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
     j.total_items = total;
     // a batch's records are moved to per-instance segments in the buffer's upper half
     j.rec_cap = std::min(ni > 1 ? ws.rec_cap / 2 : ws.rec_cap, record_capacity());
+    if (j.give_up_records)
+        j.rec_cap = std::min(j.rec_cap, j.give_up_records);
     int bps = scan_blocks_per_sm(j.acc, j.K <= 1, j.variant);
     if (bps < 1)
         bps = 1;
@@ -693,6 +696,7 @@ int job_enqueue_scan(Workspace &ws, Job &j, const void *state_init = nullptr)
         a.margin += acc_float(j.acc) ? j.window : std::floor(j.window);
     a.zero = 0;
     a.mad_inverse = kMadInverse;
+    a.give_up = j.give_up_records ? 1 : 0;
     CK(launch_scan(j.acc, a, j.blocks, j.variant, s));
     CK(record_event(ws.ev[1], s));
     j.launches += 2;
@@ -938,6 +942,7 @@ struct SolveCfg {
     double time_limit = 0.0;
     int split_k = 0, walk_bits = 0;
     int variant = -1;  // < 0: the accumulator's default (or QUBO_SCAN_VARIANT)
+    unsigned long long give_up_records = 0;  // > 0: the run ends (Part::overflow) past so many candidates
 };
 
 struct SolveStats {
@@ -979,8 +984,11 @@ int solve_range(Workspace &ws, HostInst &h, int fix_bits, uint64_t fix_value, co
     j.variant = h.variant;
     j.stream = stream;
     j.window = c.window;
+    j.give_up_records = c.give_up_records;
     if ((st = job_launch(ws, j)))
         return st;
+    if (h.acc == ACC_F32 && !h.small)
+        fp32_bound_terms(h);  // reported with the result; formed while the scan runs
     std::vector<Part> parts;
     double gs = 0.0;
     st = job_finish(ws, j, parts, &gs);
@@ -988,7 +996,7 @@ int solve_range(Workspace &ws, HostInst &h, int fix_bits, uint64_t fix_value, co
     if (st)
         return st;
     Part p = parts[0];
-    if (!p.overflow) {
+    if (!p.overflow || c.give_up_records) {
         out = p;
         return QUBO_OK;
     }
@@ -1008,13 +1016,49 @@ int solve_range(Workspace &ws, HostInst &h, int fix_bits, uint64_t fix_value, co
 // FP32 scans: the candidate margin must cover twice the measured drift plus the rounding of the
 // per-step threshold arithmetic (a few FP32 operations on values bounded by beta; the factored
 // scan's E_L plus up to 14 zero-row couplings, more).  Otherwise the caller rescans with a
-// shorter walk, the dense FP32 scan, or FP64.
+// shorter walk, the dense FP32 scan, a proven margin, or FP64.  Direct evaluation sums in FP64.
+double float_slack(const HostInst &h)
+{
+    return (h.acc == ACC_F32Z ? 32.0 : 8.0) * std::ldexp(1.0, -24) * (1.0 + h.beta);
+}
 bool float_margin_ok(const HostInst &h, const Part &p, double margin)
 {
-    if (h.acc != ACC_F32 && h.acc != ACC_F32Z)
+    if ((h.acc != ACC_F32 && h.acc != ACC_F32Z) || h.small)
         return true;
-    const double slack = (h.acc == ACC_F32Z ? 32.0 : 8.0) * std::ldexp(1.0, -24) * (1.0 + h.beta);
-    return 2.0 * p.drift + slack < margin;
+    return 2.0 * p.drift + float_slack(h) < margin;
+}
+
+// A float instance whose magnitudes leave the caller's candidate margin no room for an FP32 scan's
+// rounding (entries of order 100 at n = 30) is scanned in FP32 all the same, with a wider margin: twice
+// the worst-case rounding bound of the run's plan, which proves that every state of the answer reaches
+// the FP64 rescoring.  A wider margin only adds candidates.  When they are more than kProvenRecords
+// (dense low spectra, e.g. large penalty terms) the run ends early and the FP64 scan runs instead, as
+// without this attempt.  n=31, entries uniform in [-100, 100]: 0.19 ms of scan against 9.2 ms in FP64
+// (an FP64 add takes a warp 70 cycles on GB300), which three FP32 scans preceded.
+constexpr unsigned long long kProvenRecords = 1ull << 16;
+int solve_proven(Workspace &ws, HostInst &h, const qubo_options &o, SolveCfg c, cudaStream_t stream, Part &p,
+                 SolveStats &stats, double deadline, bool *done)
+{
+    *done = false;
+    if (!(h.beta < 1e30))  // FP32 range
+        return QUBO_OK;
+    h.acc = ACC_F32;
+    h.no_factored = true;
+    int st = plan_run(h, o.fix_bits, o.fix_value, c.split_k, c.walk_bits, c.variant, c.flags, c.margin);
+    if (st || h.acc != ACC_F32 || h.small)
+        return st;
+    h.anchor_bits = std::max(variant_reg_rows(h) + 1, std::min(h.anchor_bits, h.L));
+    // the bound's threshold terms carry the margin itself (a few 2^-24 of it)
+    const double m = 2.0 * fp32_error_bound(h, h.anchor_bits, c.margin) * 1.0001;
+    if (!(m > c.margin) || 2.0 * fp32_error_bound(h, h.anchor_bits, m) > m)
+        return QUBO_OK;
+    c.margin = m;
+    c.give_up_records = kProvenRecords;
+    p = Part();
+    if ((st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))
+        return st;
+    *done = !p.overflow && h.acc == ACC_F32 && float_margin_ok(h, p, m);
+    return QUBO_OK;
 }
 
 void fill_outputs(const HostInst &h, const Part &p, int K, size_t cap, void *out_min, uint64_t *out_states,
@@ -1115,12 +1159,21 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
 {
     SolveCfg c = solve_cfg(h, o, states_cap, window);
     const double deadline = o.time_limit_s > 0 ? now_s() + o.time_limit_s : 0.0;
-    int st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline);
-    if (st)
+    int st;
+    const bool fp32 = h.acc == ACC_F32 && !(c.flags & (QUBO_FLAG_PLAIN | QUBO_FLAG_RIGOROUS));
+    bool done = false, tried = false;
+    if (fp32 && !(float_slack(h) < c.margin)) {  // no drift, however small, would fit the margin
+        tried = true;
+        if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
+            return st;
+        if (!done && !h.small)
+            h.acc = ACC_F64;
+    }
+    if (!done && (st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))
         return st;
-    // FP32 drift above the margin's budget: shorten the re-anchoring period, and as a last resort
-    // rescan in FP64.
-    while (!float_margin_ok(h, p, c.margin)) {
+    // FP32 drift above the margin's budget: shorten the re-anchoring period, then take a proven
+    // margin, and as a last resort rescan in FP64.
+    while (!done && !float_margin_ok(h, p, c.margin)) {
         const int period = std::min(h.anchor_bits, h.L);
         if (h.acc == ACC_F32Z) {  // the dense FP32 scan next
             h.no_factored = true;
@@ -1129,6 +1182,13 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
         } else if (h.acc == ACC_F32 && !h.small && period > variant_reg_rows(h) + 1) {
             h.anchor_bits = std::max(variant_reg_rows(h) + 1, period - 2);
         } else {
+            if (fp32 && !tried) {
+                tried = true;
+                if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
+                    return st;
+                if (done)
+                    break;
+            }
             h.acc = ACC_F64;
             c.walk_bits = o.walk_bits;
         }
@@ -1143,6 +1203,14 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
     if (p.scanned != expect || !p.has)
         return QUBO_ERR_INTERNAL;
     return QUBO_OK;
+}
+
+// A batched instance solved again alone because its FP32 margin does not hold.
+int solve_alone(Workspace &ws, HostInst &h, int topk, size_t cap, cudaStream_t stream, Part &p, SolveStats &stats)
+{
+    qubo_options o{};
+    o.topk = topk;
+    return solve_one(ws, h, o, cap, stream, p, stats);
 }
 
 void fill_plan_info(const HostInst &h, const SolveStats &stats, double t0, qubo_result *info)
@@ -1399,11 +1467,12 @@ int batch_parts(Workspace &ws, std::vector<HostInst> &hs, const std::vector<int>
         Part &p = run_parts[r];
         HostInst &h = hs[i];
         if (p.overflow || !float_margin_ok(h, p, c.margin)) {
-            // rare: this instance overflowed the shared candidate buffer; solve it alone
-            if (!float_margin_ok(h, p, c.margin))
-                h.acc = ACC_F64;
+            // rare: this instance overflowed the shared candidate buffer, or its FP32 margin does not
+            // hold; solve it alone
+            const bool overflow = p.overflow;
             p = Part();
-            if ((st = solve_range(ws, h, 0, 0, c, stream, p, stats, 0.0)))
+            if ((st = overflow ? solve_range(ws, h, 0, 0, c, stream, p, stats, 0.0)
+                               : solve_alone(ws, h, topk, cap, stream, p, stats)))
                 return st;
         }
         if (p.scanned != (1ull << h.n) || !p.has)
@@ -2253,10 +2322,10 @@ int qubo_batch_fetch(qubo_batch *b, void *out_min, uint64_t *out_states, uint64_
             if ((st = sw->init(dev)))
                 return st;
             HostInst hc = h;
-            if (!float_margin_ok(hc, p, c.margin))
-                hc.acc = ACC_F64;
+            const bool overflow = p.overflow;
             p = Part();
-            if ((st = solve_range(*sw, hc, 0, 0, c, j.stream, p, st2, 0.0)))
+            if ((st = overflow ? solve_range(*sw, hc, 0, 0, c, j.stream, p, st2, 0.0)
+                               : solve_alone(*sw, hc, b->topk, b->cap, j.stream, p, st2)))
                 return st;
         }
         if (p.scanned != (1ull << h.n) || !p.has)

@@ -47,8 +47,7 @@ inline double now_s()
 struct Fp32BoundTerms {
     bool valid = false;
     int n = 0, B = 0, L = 0, rc = 0;
-    double margin = 0.0;
-    double Cc = 0.0, CP = 0.0, Ecol0 = 0.0, EP0 = 0.0, rest = 0.0;
+    double Cc = 0.0, CP = 0.0, Ecol0 = 0.0, EP0 = 0.0, rest = 0.0;  // rest: without the margin's part
 };
 
 // One instance prepared on the host and the plan of its current run.
@@ -132,7 +131,7 @@ double threshold_bound(const HostInst &h, int K, int restarts = 24);
 // Dense FP32 scan: worst-case rounding error of a state's decision value at a re-anchoring period
 // of 2^anchor_bits walk steps, and the longest period whose bound alone guarantees the candidates
 // (2 bound <= margin; -1 if none).  0 / -1 for other accumulators.
-const Fp32BoundTerms &fp32_bound_terms(const HostInst &h, double margin);
+const Fp32BoundTerms &fp32_bound_terms(const HostInst &h);
 double fp32_error_bound(const HostInst &h, int anchor_bits, double margin);
 int fp32_rigorous_anchor_bits(const HostInst &h, double margin);
 

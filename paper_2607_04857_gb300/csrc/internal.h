@@ -195,6 +195,7 @@ struct ScanArgs {
     const volatile int *abort_flag;
     double margin;               // float scans: candidate margin above the threshold
     int32_t zero;                // the constant 0, passed at run time (packed 3-input-add variants)
+    int32_t give_up;             // end the scan once more candidates were offered than rec_cap
     uint32_t mad_inverse;        // kMadInverse, passed at run time (integer updates of the grouped form)
 };
 

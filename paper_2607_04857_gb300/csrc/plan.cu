@@ -805,12 +805,13 @@ namespace host {
 // A state x of the answer has E(x) <= E(y) for the state y whose
 // computed energy set the threshold, so it is recorded whenever 2 Edec <= margin; its FP64
 // rescoring then decides.  The bound is a worst case over every state of the run.
-// The plan-dependent magnitudes of the bound, computed once per (B, L, RC, margin) and kept in h.
-const Fp32BoundTerms &fp32_bound_terms(const HostInst &h, double margin)
+// The plan-dependent magnitudes of the bound, computed once per (B, L, RC) and kept in h; the margin
+// enters CT alone (three times u).
+const Fp32BoundTerms &fp32_bound_terms(const HostInst &h)
 {
     Fp32BoundTerms &m = h.fp32_terms;
     const int rc = variant_reg_rows(h);
-    if (m.valid && m.B == h.B && m.L == h.L && m.rc == rc && m.n == h.n && m.margin == margin)
+    if (m.valid && m.B == h.B && m.L == h.L && m.rc == rc && m.n == h.n)
         return m;
     const int n = h.n, B = h.B, L = h.L, k = h.k, nf = B + L;
     const double u = std::ldexp(1.0, -24);
@@ -879,7 +880,7 @@ const Fp32BoundTerms &fp32_bound_terms(const HostInst &h, double margin)
         // the walk's own rounding is far below the slack of the bound; widen by it anyway
         CL *= 1.0 + std::ldexp(1.0, -30);
     }
-    const double CT = beta * (1.0 + std::ldexp(1.0, -20)) + margin;
+    const double CT = beta * (1.0 + std::ldexp(1.0, -20));
     const double e64 = (double)n * n * std::ldexp(1.0, -52) * beta;
     const double u64 = std::ldexp(1.0, -52);
     double Ecol0 = 2 * u * Cc + e64 + (B + 3) * u * CabsF + k * u64 * CabsF + (L - rc) * u * Cc;
@@ -893,7 +894,6 @@ const Fp32BoundTerms &fp32_bound_terms(const HostInst &h, double margin)
     m.B = B;
     m.L = L;
     m.rc = rc;
-    m.margin = margin;
     m.Cc = Cc;
     m.CP = CP;
     m.Ecol0 = Ecol0;
@@ -906,13 +906,13 @@ double fp32_error_bound(const HostInst &h, int anchor_bits, double margin)
 {
     if (h.acc != ACC_F32 || h.small || h.Uf.empty())
         return 0.0;
-    const Fp32BoundTerms &m = fp32_bound_terms(h, margin);
+    const Fp32BoundTerms &m = fp32_bound_terms(h);
     const double u = std::ldexp(1.0, -24);
     const int a = std::min(std::max(anchor_bits, m.rc + 1), m.L);
     const double Ecol = m.Ecol0 + std::expm1(std::ldexp(1.0, a) * std::log1p(u)) * (m.Cc + m.Ecol0);
     const double tP = std::ldexp(1.0, std::max(0, a - m.rc - 1)) + 1.0;
     const double EP = m.EP0 + std::expm1(tP * std::log1p(u)) * (m.CP + m.EP0);
-    return Ecol + (m.rc + 1) * u * (m.Cc + Ecol) + EP + m.rest;
+    return Ecol + (m.rc + 1) * u * (m.Cc + Ecol) + EP + m.rest + 3.0 * u * margin;
 }
 
 // Longest re-anchoring period (log2 of walk steps, from one unrolled body up to the whole walk)

@@ -398,6 +398,8 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
         for (int p = 0; p < BODY; ++p) {
             if (!((hits >> (p >> 4)) & 1u))
                 continue;
+            if (Tr<T>::kFloat && gave_up(a))
+                break;
             const int i = i0 + p, gp = i ^ (i >> 1);
             TC sr[NR], least{};
 #pragma unroll

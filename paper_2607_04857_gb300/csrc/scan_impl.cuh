@@ -331,6 +331,12 @@ __device__ __forceinline__ T tree_min(const T (&E)[N])
     }
 }
 
+// Whether a run that gives up past its buffer's capacity (ScanArgs::give_up) has reached it.
+__device__ __forceinline__ bool gave_up(const ScanArgs &a)
+{
+    return a.give_up && *(const volatile unsigned long long *)a.nrec > a.rec_cap;
+}
+
 // Offer one state to the candidate buffer.
 template <class T>
 __device__ __forceinline__ void record(const ScanArgs &a, int inst, typename Tr<T>::TP E, uint64_t code)
@@ -1236,7 +1242,7 @@ __device__ __forceinline__ void persistent_units(const ScanArgs &a, int lane, ty
         unsigned long long base = 0;
         int stop = 0;
         if (lane == 0) {
-            stop = *a.abort_flag != 0;
+            stop = *a.abort_flag != 0 || gave_up(a);
             base = next;
             if (!stop && base < a.total_items)
                 next = atomicAdd(a.queue, kChunk);

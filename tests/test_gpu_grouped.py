@@ -156,3 +156,43 @@ def test_record_list_lengths(q, zeros):
     assert r.min == o.min and r.n_ties == o.n_ties and np.array_equal(r.ties, o.ties) and np.array_equal(r.topk, o.topk)
     for r, e in zip(q.solve_batched([few.astype(np.float32), F], topk=30, states_cap=5000), (of, o)):
         assert r.min == e.min and r.n_ties == e.n_ties and np.array_equal(r.ties, e.ties)
+
+
+# --- float magnitudes beyond the caller's margin -------------------------------------------------
+
+def check_exact_float(r, o):
+    assert r.min == o.min and r.n_ties == o.n_ties
+    assert np.array_equal(r.ties, o.ties) and np.array_equal(r.topk, o.topk) and np.array_equal(r.topk_E, o.topk_E)
+
+
+@pytest.mark.parametrize("scale", [1.0, 30.0, 100.0, 1e6, 1e20, 1e35])
+@pytest.mark.parametrize("n", [14, 20, 26])
+def test_float_proven_margin(q, n, scale):
+    """Entries from where the default margin holds to where no FP32 scan can run: FP32 with a proven
+    margin up to FP32's range (every returned energy the FP64 sum), FP64 beyond it."""
+    rng = np.random.default_rng(n)
+    Q = rng.uniform(-scale, scale, (n, n))
+    r, o = q.solve(Q, topk=10), oracle.solve(Q, topk=10)
+    check_exact_float(r, o)
+    assert r.info["acc"] == ("f64" if scale > 1e30 else "f32"), r.info
+    if r.info["acc"] == "f32" and scale >= 100 and n > 14:
+        assert r.info["passes"] == 1
+    rs = q.solve_batched([Q, Q / scale], topk=10)
+    check_exact_float(rs[0], o)
+
+
+def test_float_proven_margin_gives_up(q):
+    """A penalty encoding: 2^16 and more states within the proven margin of the minimum; the attempt
+    ends early and the FP64 scan decides."""
+    n = 22
+    Q = np.zeros((n, n))
+    Q[0, 0] = 1e7
+    Q[np.arange(1, n), np.arange(1, n)] = np.random.default_rng(1).uniform(-1e-3, 1e-3, n - 1)
+    Q[1, 2] = 1e-4
+    r = q.solve(Q, topk=16)
+    assert r.info["acc"] == "f64" and r.info["passes"] >= 2, r.info
+    check_exact_float(r, oracle.solve(Q, topk=16))
+    cnt, codes, E, _ = q.solve_window(Q, 2e-4)
+    o = oracle.solve(Q, topk=4096, cap=1)
+    sel = o.topk_E <= o.min + 2e-4
+    assert not sel.all() and cnt == int(sel.sum()) and np.array_equal(codes, o.topk[sel])
