@@ -145,7 +145,7 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
     constexpr int LOGV = ilog2c(V), LOGG = ilog2c(G);
     constexpr int B = LOGV + 5 + LOGG, NB = 1 << B;
     static_assert((RC == 4 && NG == 1) || (RC == 5 && NG == 4), "a body's flips below row RC are register rows");
-    constexpr int NR = 4 + ilog2c(NG);  // register rows a body flips
+    constexpr int NR = 4 + ilog2c(NG);  // rows a body flips
     const int n = d.n, L = d.L, k = d.k, BL = B + L;
     InstState *st = a.state + inst;
 
@@ -388,64 +388,126 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
         }
     };
 
-    // Rare: rebuild every state of the body's groups in hits from the body's last state (which
-    // differs by the register rows, and with NG > 1 row RC, whose Gray bits differ) and record each
-    // column at or below the threshold.  Pmid: P before the flip of row RC.
-    auto record_hits = [&](int i0, unsigned hits, TP Pmid) {
-        const int iend = i0 + BODY - 1, gend = iend ^ (iend >> 1);
-        const TC *rowRC = Mt + (size_t)RC * NB;
+    // Rare: offer the staged columns of walk step i (P = Pp, E_L = elp) at or below the threshold tp.
+    auto record_staged = [&](int i, TP Pp, TC elp, TC tp) {
+        const uint64_t cb = cbase | ((uint64_t)(i ^ (i >> 1)) << B);
+        const TP Ep = Pp + (TP)elp;
 #pragma unroll 1
-        for (int p = 0; p < BODY; ++p) {
-            if (!((hits >> (p >> 4)) & 1u))
-                continue;
-            if (Tr<T>::kFloat && gave_up(a))
-                break;
-            const int i = i0 + p, gp = i ^ (i >> 1);
-            TC sr[NR], least{};
-#pragma unroll
-            for (int r = 0; r < NR; ++r)
-                sr[r] = r < RC ? (TC)(((gp >> r) & 1) - ((gend >> r) & 1)) : (TC)0;
-            const int dRC = NG == 4 ? ((gp >> RC) & 1) - ((gend >> RC) & 1) : 0;
-            const TC sRC = (TC)dRC;
-            const TP Pp = dRC == 0 ? P : Pmid;
-            const TC elp = ELp[i];
-            TC tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                TC mv[V];
-                if constexpr (NG == 4)
-                    vload<TC>(rowRC + (g * 32 + lane) * V, mv);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    const int q = g * V + e;
-                    TC x = E[q];
-#pragma unroll
-                    for (int r = 0; r < NR && r < RC; ++r)
-                        x = x + sr[r] * mad_factor<TC>(r, q) * Mr[r][q];
-                    if constexpr (NG == 4)
-                        x = x + sRC * mv[e];
-                    stage[q * 32 + lane] = x;
-                    least = q == 0 ? x : emin(least, x);
+        for (int q = 0; q < S; ++q) {
+            const TC v = stage[q * 32 + lane];
+            if (v <= tp) {
+                const TP Et = (TP)v + Ep;
+                const uint32_t j = (uint32_t)(((q / V) * 32 + lane) * V + (q % V));
+                record<T>(a, inst, Et, cb | j);
+                if (K1 && Et < Treg) {
+                    Treg = Et;
+                    tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
+                    Tr<T>::thr_min(st, Et);
                 }
             }
-            if (!(least <= tp))
-                continue;
-            const uint64_t cb = cbase | ((uint64_t)gp << B);
-            const TP Ep = Pp + (TP)elp;
+        }
+    };
+    // Columns of walk step i of the body from those of step j: the register rows, and with NG > 1 row
+    // RC, whose Gray bits differ.
+    const TC *rowRC = Mt + (size_t)RC * NB;
+    [[maybe_unused]] auto move = [&](TC (&x)[S], int i, int j) {
+        const int gi = i ^ (i >> 1), gj = j ^ (j >> 1);
+        TC sr[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            sr[r] = (TC)(((gi >> r) & 1) - ((gj >> r) & 1));
+        static_for<G>([&](auto gc) {
+            constexpr int g = decltype(gc)::value;
+            TC mv[V];
+            if constexpr (NG > 1)
+                vload<TC>(rowRC + (g * 32 + lane) * V, mv);
+            static_for<V>([&](auto ec) {
+                constexpr int e = decltype(ec)::value, q = g * V + e;
+                static_for<(NR < RC ? NR : RC)>([&](auto rc) {
+                    constexpr int r = decltype(rc)::value;
+                    x[q] = x[q] + sr[r] * mad_factor<TC>(r, q) * Mr[r][q];
+                });
+                if constexpr (NG > 1)
+                    x[q] = x[q] + sr[RC] * mv[e];
+            });
+        });
+    };
+    // The states of the body's groups in hits, E being the body's last one.  Integer columns (exact)
+    // are moved to each group's first state, walked through it and moved back; FP32 columns are
+    // left alone and every state is rebuilt from the last one.  Pmid: P before the flip of row RC.
+    auto record_hits = [&](int i0, unsigned hits, TP Pmid) {
+        const int iend = i0 + BODY - 1;
+        auto prefix = [&](int i) {
+            return NG == 1 || (((i ^ (i >> 1)) ^ (iend ^ (iend >> 1))) >> RC & 1) == 0 ? P : Pmid;
+        };
+        if constexpr (Tr<T>::kFloat) {
+            const int gend = iend ^ (iend >> 1);
 #pragma unroll 1
-            for (int q = 0; q < S; ++q) {
-                const TC x = stage[q * 32 + lane];
-                if (x <= tp) {
-                    const TP Et = (TP)x + Ep;
-                    const uint32_t j = (uint32_t)(((q / V) * 32 + lane) * V + (q % V));
-                    record<T>(a, inst, Et, cb | j);
-                    if (K1 && Et < Treg) {
-                        Treg = Et;
-                        tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
-                        Tr<T>::thr_min(st, Et);
+            for (int p = 0; p < BODY; ++p) {
+                if (!((hits >> (p >> 4)) & 1u))
+                    continue;
+                if (gave_up(a))
+                    break;
+                const int i = i0 + p, gp = i ^ (i >> 1);
+                TC sr[NR], least{};
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    sr[r] = (TC)(((gp >> r) & 1) - ((gend >> r) & 1));
+                const TP Pp = prefix(i);
+                const TC elp = ELp[i];
+                TC tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    TC mv[V];
+                    if constexpr (NG > 1)
+                        vload<TC>(rowRC + (g * 32 + lane) * V, mv);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) {
+                        const int q = g * V + e;
+                        TC x = E[q];
+#pragma unroll
+                        for (int r = 0; r < NR && r < RC; ++r)
+                            x = x + sr[r] * Mr[r][q];
+                        if constexpr (NG > 1)
+                            x = x + sr[RC] * mv[e];
+                        stage[q * 32 + lane] = x;
+                        least = q == 0 ? x : emin(least, x);
                     }
                 }
+                if (least <= tp)
+                    record_staged(i, Pp, elp, tp);
             }
+        } else {
+            int at = iend;
+#pragma unroll 1
+            for (int p = 0; p < BODY; ++p) {
+                if (!((hits >> (p >> 4)) & 1u))
+                    continue;
+                if (p % 16 == 0) {
+                    move(E, i0 + p, at);
+                } else {
+                    const int row = __ffs(p) - 1;
+                    const TC sg = ((p + i0) >> (row + 1)) & 1 ? (TC)-1 : (TC)1;
+                    static_for<4>([&](auto rc) {
+                        constexpr int r = decltype(rc)::value;
+                        if (row == r)
+                            static_for<S>([&](auto qc) {
+                                constexpr int q = decltype(qc)::value;
+                                E[q] = E[q] + sg * mad_factor<TC>(r, q) * Mr[r][q];
+                            });
+                    });
+                }
+                at = i0 + p;
+                const TP Pp = prefix(at);
+                const TC elp = ELp[at], tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
+                if (!(tree_min<TC, 3, S>(E) <= tp))
+                    continue;
+#pragma unroll
+                for (int q = 0; q < S; ++q)
+                    stage[q * 32 + lane] = E[q];
+                record_staged(at, Pp, elp, tp);
+            }
+            move(E, iend, at);
         }
         u = Treg + mu - P;
         uc = to_col<T>(u, clampC);
@@ -650,61 +712,81 @@ __device__ __forceinline__ void scan_unit_packed_grouped(const ScanArgs &a, cons
     };
 
     constexpr int LOGBODY = 4 + ilog2c(NG), BODY = 1 << LOGBODY;
+    auto record_state = [&](int i, int32_t Pp) {
+        const int32_t els = ELp[i];
+        int32_t tp = Treg + mu - Pp - els;
+        if (lane_min(tree_min<uint32_t, 3, S>(E)) > tp)
+            return;
+#pragma unroll
+        for (int q = 0; q < S; ++q)
+            stage[q * 32 + lane] = E[q];
+        const uint64_t cb = cbase | ((uint64_t)(i ^ (i >> 1)) << B);
+#pragma unroll 1
+        for (int q = 0; q < 2 * S; ++q) {
+            const int qw = q >> 1;
+            const uint32_t word = stage[qw * 32 + lane];
+            const int32_t x = (int32_t)((q & 1) ? (word >> 16) : (word & 0xffffu));
+            if (x <= tp) {
+                const int32_t Et = x + els + Pp;
+                const uint32_t j = (uint32_t)(((qw / V) * 32 + lane) * V + (qw % V)) + ((q & 1) ? NW : 0);
+                record<T>(a, inst, Et, cb | j);
+                if (K1 && Et < Treg) {
+                    Treg = Et;
+                    tp = Treg + mu - Pp - els;
+                    Tr<T>::thr_min(st, Et);
+                }
+            }
+        }
+    };
+    const uint32_t *rowRC = Mt + (size_t)RC * NW;
+    auto move = [&](int i, int j) {
+        const int gi = i ^ (i >> 1), gj = j ^ (j >> 1);
+        uint32_t sr[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            sr[r] = (uint32_t)(((gi >> r) & 1) - ((gj >> r) & 1));
+        static_for<G>([&](auto gc) {
+            constexpr int g = decltype(gc)::value;
+            uint32_t mv[V];
+            if constexpr (NG > 1)
+                vload<uint32_t>(rowRC + (g * 32 + lane) * V, mv);
+            static_for<V>([&](auto ec) {
+                constexpr int e = decltype(ec)::value, q = g * V + e;
+                static_for<(NR < RC ? NR : RC)>([&](auto rc) {
+                    constexpr int r = decltype(rc)::value;
+                    E[q] += sr[r] * mad_factor<uint32_t>(r, q) * Mr[r][q];
+                });
+                if constexpr (NG > 1)
+                    E[q] += sr[RC] * mv[e];
+            });
+        });
+    };
     auto record_hits = [&](int i0, unsigned hits, int32_t Pmid) {
-        const int iend = i0 + BODY - 1, gend = iend ^ (iend >> 1);
-        const uint32_t *rowRC = Mt + (size_t)RC * NW;
+        const int iend = i0 + BODY - 1;
+        int at = iend;
 #pragma unroll 1
         for (int p = 0; p < BODY; ++p) {
             if (!((hits >> (p >> 4)) & 1u))
                 continue;
-            const int i = i0 + p, gp = i ^ (i >> 1);
-            uint32_t sr[NR];
-#pragma unroll
-            for (int r = 0; r < NR; ++r)
-                sr[r] = r < RC ? (uint32_t)(((gp >> r) & 1) - ((gend >> r) & 1)) : 0u;
-            const int dRC = NG == 4 ? ((gp >> RC) & 1) - ((gend >> RC) & 1) : 0;
-            const int32_t Pp = dRC == 0 ? P : Pmid;
-            const int32_t els = ELp[i];
-            int32_t tp = Treg + mu - Pp - els;
-            uint32_t least = ~0u;
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                uint32_t mv[V];
-                if constexpr (NG == 4)
-                    vload<uint32_t>(rowRC + (g * 32 + lane) * V, mv);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    const int q = g * V + e;
-                    uint32_t x = E[q];
-#pragma unroll
-                    for (int r = 0; r < NR && r < RC; ++r)
-                        x += sr[r] * mad_factor<uint32_t>(r, q) * Mr[r][q];
-                    if constexpr (NG == 4)
-                        x += (uint32_t)dRC * mv[e];
-                    stage[q * 32 + lane] = x;
-                    least = __vminu2(least, x);
-                }
+            if (p % 16 == 0) {
+                move(i0 + p, at);
+            } else {
+                const int row = __ffs(p) - 1;
+                const uint32_t sg = ((p + i0) >> (row + 1)) & 1 ? ~0u : 1u;
+                static_for<4>([&](auto rc) {
+                    constexpr int r = decltype(rc)::value;
+                    if (row == r)
+                        static_for<S>([&](auto qc) {
+                            constexpr int q = decltype(qc)::value;
+                            E[q] += sg * mad_factor<uint32_t>(r, q) * Mr[r][q];
+                        });
+                });
             }
-            if (lane_min(least) > tp)
-                continue;
-            const uint64_t cb = cbase | ((uint64_t)gp << B);
-#pragma unroll 1
-            for (int q = 0; q < 2 * S; ++q) {
-                const int qw = q >> 1;
-                const uint32_t word = stage[qw * 32 + lane];
-                const int32_t x = (int32_t)((q & 1) ? (word >> 16) : (word & 0xffffu));
-                if (x <= tp) {
-                    const int32_t Et = x + els + Pp;
-                    const uint32_t j = (uint32_t)(((qw / V) * 32 + lane) * V + (qw % V)) + ((q & 1) ? NW : 0);
-                    record<T>(a, inst, Et, cb | j);
-                    if (K1 && Et < Treg) {
-                        Treg = Et;
-                        tp = Treg + mu - Pp - els;
-                        Tr<T>::thr_min(st, Et);
-                    }
-                }
-            }
+            at = i0 + p;
+            const int ga = at ^ (at >> 1), ge = iend ^ (iend >> 1);
+            record_state(at, NG == 1 || ((ga ^ ge) >> RC & 1) == 0 ? P : Pmid);
         }
+        move(iend, at);
         u = Treg + mu - P;
     };
 
