@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 from dataclasses import dataclass, field
 
 import numpy as np
@@ -175,14 +176,11 @@ def abort_clear() -> None:
 
 def _stream_ptr(stream):
     """cudaStream_t as an integer: an int, an object with .cuda_stream (torch), or the current
-    torch stream when torch with CUDA is available; else the default stream."""
+    torch stream when torch with CUDA is in use; else the default stream."""
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return int(torch.cuda.current_stream().cuda_stream)
-        except ImportError:
-            pass
+        torch = sys.modules.get("torch")  # a process that has not imported it has no current torch stream
+        if torch is not None and torch.cuda.is_initialized():
+            return int(torch.cuda.current_stream().cuda_stream)
         return None
     if hasattr(stream, "cuda_stream"):
         return int(stream.cuda_stream)

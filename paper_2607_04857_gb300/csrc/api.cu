@@ -219,6 +219,7 @@ struct Workspace {
     int *h_abort = nullptr;        // host-mapped flag read by the scan kernel
     const int *d_abort = nullptr;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // tables start, scan end, finalize end, scan start
+    std::map<std::tuple<int, bool, int>, int> blocks_per_sm;  // scan_blocks_per_sm on this device, as asked for
     std::mutex mu;
 
     ~Workspace() { release(); }
@@ -249,6 +250,7 @@ struct Workspace {
         d_rec = nullptr;
         h_up = h_down = nullptr;
         h_abort = nullptr;
+        blocks_per_sm.clear();
         dev = -1;
     }
 
@@ -651,9 +653,9 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
     j.rec_cap = std::min(ni > 1 ? ws.rec_cap / 2 : ws.rec_cap, record_capacity());
     if (j.give_up_records)
         j.rec_cap = std::min(j.rec_cap, j.give_up_records);
-    int bps = scan_blocks_per_sm(j.acc, j.K <= 1, j.variant);
+    int &bps = ws.blocks_per_sm[{(int)j.acc, j.K <= 1, j.variant}];
     if (bps < 1)
-        bps = 1;
+        bps = std::max(1, scan_blocks_per_sm(j.acc, j.K <= 1, j.variant));
     j.blocks = ws.sms * bps;
     const uint64_t need_blocks = (total * 32 + kScanThreads - 1) / kScanThreads;
     if ((uint64_t)j.blocks > need_blocks)
@@ -718,9 +720,12 @@ int job_launch(Workspace &ws, Job &j)
     return QUBO_OK;
 }
 
-// Wait for `ev` (the run's end), honouring the time limit and qubo_abort.
+// Wait for `ev` (the run's end), honouring the time limit and qubo_abort.  The event is polled without a
+// pause for the first 2 ms (a pause of 200 us, as the kernel's timer slack makes it, was 60% of a small
+// solve), then at intervals of 1/200 of the time waited, 20 to 200 us.
 int job_wait(Workspace &ws, Job &j, cudaEvent_t ev)
 {
+    const double t0 = now_s();
     for (;;) {
         const cudaError_t q = cudaEventQuery(ev);
         if (q == cudaSuccess)
@@ -734,7 +739,9 @@ int job_wait(Workspace &ws, Job &j, cudaEvent_t ev)
             *(volatile int *)ws.h_abort = 1;
             j.aborted = true;
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(200));
+        const double waited = now_s() - t0;
+        if (waited > 2e-3)
+            std::this_thread::sleep_for(std::chrono::duration<double>(std::min(2e-4, std::max(2e-5, waited / 200))));
     }
     if (*(volatile int *)ws.h_abort)
         j.aborted = true;
@@ -1260,16 +1267,26 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order);
 // Walk length of a batched instance in (acc, variant): the walk the batch autotuner installed
 // for its size under this variant, else as long as the instance allows (at most wmax); 0 when
 // the instance is too small to split.  h.acc and h.variant must be set.
-int batch_walk(Acc acc, int variant, const HostInst &h, int wmax)
+int batch_walk(Acc acc, int variant, const HostInst &h, int wmax, const int (&tuned)[kMaxBatchedN + 1])
 {
     const int B = acc_suffix_bits(acc, variant);
     const int rmin = variant_reg_rows(h) + 1;
     if (h.n - B < rmin)
         return 0;
-    int tv = 0, tw = 0;
-    if (tuned_plan(acc, -h.n, &tv, &tw) && tv == variant && tw >= rmin && tw <= std::min(kMaxWalkBits, h.n - B))
+    const int tw = tuned[h.n];
+    if (tw >= rmin && tw <= std::min(kMaxWalkBits, h.n - B))
         return tw;
     return std::max(rmin, std::min(wmax, h.n - B));
+}
+
+// The walks installed per size for a batch in (acc, variant), 0 where none is (looked up once per
+// batch: the lookup locks).
+void batch_tuned_walks(Acc acc, int variant, int (&tuned)[kMaxBatchedN + 1])
+{
+    for (int n = 0; n <= kMaxBatchedN; ++n) {
+        int tv = 0, tw = 0;
+        tuned[n] = n > 0 && tuned_plan(acc, -n, &tv, &tw) && tv == variant ? tw : 0;
+    }
 }
 
 // Longest walk of a batch's grouped scan, up to wmax: the one whose units, shared by the resident
@@ -1354,18 +1371,20 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order)
     if (acc_bytes(acc) != 4)
         variant = 0;
     const int wmax = batch_max_walk(acc, variant, hs, acc == ACC_F32 ? kFloatMaxWalkBits : kDefaultMaxWalkBits);
+    int tuned[kMaxBatchedN + 1];
+    batch_tuned_walks(acc, variant, tuned);
     auto plan_range = [&](int lo, int hi) {
         for (int i = lo; i < hi; ++i) {
             HostInst &h = hs[i];
             h.variant = variant;
-            pst[i] = plan(h, 0, 0, 0, batch_walk(acc, h.variant, h, wmax));
+            pst[i] = plan(h, 0, 0, 0, batch_walk(acc, h.variant, h, wmax, tuned));
             // batches are many small instances: fewer descents (K = 1 thresholds also tighten on
             // the device as soon as a lower state is found)
             if (!pst[i])
                 h.thr0 = threshold_bound(h, std::max(1, topk), topk > 1 ? 16 : 6);
         }
     };
-    parallel(plan_range);
+    parallel_ranges(count, 8, plan_range);  // the thresholds are the larger part of a small batch's planning
     for (int i = 0; i < count; ++i)
         if (pst[i])
             return pst[i];
@@ -1387,13 +1406,14 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order)
         if (tuned_plan(alt_acc, 0, &tv, &tw))
             v2 = tv;
         const int wbest = batch_max_walk(alt_acc, v2, hs, alt_walk);
+        batch_tuned_walks(alt_acc, v2, tuned);
         std::atomic<bool> all{true};
         auto alt_range = [&](int lo, int hi) {
             for (int i = lo; i < hi && all.load(std::memory_order_relaxed); ++i) {
                 HostInst &h = hs[i];
                 h.acc = alt_acc;
                 h.variant = v2;
-                const bool ok = plan(h, 0, 0, 0, batch_walk(alt_acc, v2, h, wbest)) == QUBO_OK &&
+                const bool ok = plan(h, 0, 0, 0, batch_walk(alt_acc, v2, h, wbest, tuned)) == QUBO_OK &&
                                 (h.small || (alt_acc == ACC_I16P ? i16p_exact(h) : i32f_exact(h, &h.clampC)));
                 if (!ok)
                     all = false;

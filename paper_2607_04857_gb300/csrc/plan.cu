@@ -311,8 +311,12 @@ bool i32f_exact(const HostInst &h, int32_t *clampC)
     }
     int64_t lo, hi;
     col_range_exact(h, lo, hi);
-    const double el = (double)walked_energy_max(h);
-    const double C = (double)std::max(-lo, hi) + el + 1.0;
+    const double col = (double)std::max(-lo, hi);
+    if (col + 2.0 >= kLimit)
+        return false;
+    // max |E_L|: its bound S_ww when that is enough, else by enumeration
+    const double el = col + 2.0 * s_ww + 2.0 < kLimit ? s_ww : (double)walked_energy_max(h);
+    const double C = col + el + 1.0;
     if (C + el + 1.0 >= kLimit)
         return false;
     *clampC = (int32_t)C;
@@ -331,37 +335,43 @@ bool i32f_allowed()
 // with c_i(j) = sum_{b in j} U_bi, w_r = sum_{f fixed} x_f U_rf (the couplings of the register
 // rows folded into their table rows).  Its range over all outside bits is bounded by taking every
 // c_i(j) and every U_rf at its sign's extreme, computed exactly for each j (O(2^B n)).
+// The patterns are taken in Gray order with the c_i kept, in int32: the callers' beta is below 2^30.
 void col_range_exact(const HostInst &h, int64_t &lo, int64_t &hi)
 {
     const int n = h.n, B = h.B, rc = variant_reg_rows(h), nf = h.B + h.L;
-    auto U = [&](int i, int j) { return i < j ? h.Ui[(size_t)i * n + j] : h.Ui[(size_t)j * n + i]; };
+    int32_t S[64][64];  // couplings, 0 on the diagonal
+    int32_t diag[64], c[64] = {};
+    for (int i = 0; i < B; ++i) {
+        diag[i] = (int32_t)h.Ui[(size_t)i * n + i];
+        for (int j = 0; j < n; ++j)
+            S[i][j] = i == j ? 0 : (int32_t)(i < j ? h.Ui[(size_t)i * n + j] : h.Ui[(size_t)j * n + i]);
+    }
     int64_t wpos = 0, wneg = 0;
     for (int r = B; r < B + rc; ++r)
         for (int f = nf; f < n; ++f) {
-            const int64_t u = U(r, f);
+            const int64_t u = h.Ui[(size_t)r * n + f];
             (u > 0 ? wpos : wneg) += u;
         }
-    // c[j][i] for every variable i, built from j without its lowest bit
-    const size_t NB = 1ull << B;
-    std::vector<int64_t> c(NB * n, 0), es(NB, 0);
-    lo = 0;
-    hi = 0;
-    for (size_t j = 1; j < NB; ++j) {
-        const int b = __builtin_ctzll(j);
-        const size_t jp = j & (j - 1);
-        const int64_t *cp = &c[jp * n];
-        int64_t *cj = &c[j * n];
-        for (int i = 0; i < n; ++i)
-            cj[i] = cp[i] + (i == b ? 0 : U(b, i));
-        es[j] = es[jp] + U(b, b) + cp[b];
-        int64_t up = es[j], dn = es[j];
-        for (int i = B; i < n; ++i)
-            (cj[i] > 0 ? up : dn) += cj[i];
-        lo = std::min(lo, dn);
-        hi = std::max(hi, up);
+    int32_t es = 0, least = 0, most = 0;
+    for (uint32_t t = 1; t < (1u << B); ++t) {
+        const int b = __builtin_ctz(t);
+        const bool set = (((t ^ (t >> 1)) >> b) & 1) != 0;
+        const int32_t sg = set ? 1 : -1;
+        es += sg * (diag[b] + c[b]);
+        int32_t up = es, dn = es;
+        for (int i = 0; i < B; ++i)
+            c[i] += sg * S[b][i];
+        for (int i = B; i < n; ++i) {
+            const int32_t v = c[i] + sg * S[b][i];
+            c[i] = v;
+            up += v > 0 ? v : 0;
+            dn += v < 0 ? v : 0;
+        }
+        least = std::min(least, dn);
+        most = std::max(most, up);
     }
-    lo += wneg;
-    hi += wpos;
+    lo = least + wneg;
+    hi = most + wpos;
 }
 
 // Largest |E_L(g)| over the 2^L walked patterns (the energy of the walked variables alone),
@@ -682,55 +692,39 @@ double threshold_bound(const HostInst &h, int K, int restarts)
     const int n = h.n, fb = h.fix_bits, free_bits = n - fb;
     const uint64_t base = fb ? (h.fix_value << free_bits) : 0;
     const uint64_t fmask = free_bits >= 64 ? ~0ull : ((1ull << free_bits) - 1);
-    auto U = [&](int i, int j) -> double {
-        if (i > j)
-            std::swap(i, j);
-        return h.is_float ? h.Uf[(size_t)i * n + j] : (double)h.Ui[(size_t)i * n + j];
-    };
-    auto energy = [&](uint64_t x) {
-        double acc = 0.0;
-        for (int i = 0; i < n; ++i) {
-            if (!((x >> i) & 1))
-                continue;
-            acc += U(i, i);
-            for (int j = i + 1; j < n; ++j)
-                if ((x >> j) & 1)
-                    acc += U(i, j);
-        }
-        return acc;
-    };
+    // symmetric couplings, 0 on the diagonal, and the diagonal; g[v] = U_vv + field of the set bits
+    double S[64][64], diag[64], g[64], sgn[64];  // sgn: move of bit v, +1 when it is clear
+    for (int i = 0; i < n; ++i) {
+        for (int j = i; j < n; ++j)
+            S[i][j] = S[j][i] = h.is_float ? h.Uf[(size_t)i * n + j] : (double)h.Ui[(size_t)i * n + j];
+        diag[i] = S[i][i];
+        S[i][i] = 0.0;
+    }
+    K = std::max(K, 1);
     std::vector<std::pair<double, uint64_t>> seen;
-    std::unordered_set<uint64_t> codes;
+    if (K > 1)
+        seen.reserve((size_t)restarts * (free_bits + 1));
     double best1 = std::numeric_limits<double>::infinity();  // K = 1: the lowest state met
     uint64_t best1_x = 0;
-    auto offer = [&](double E, uint64_t x) {
-        if (K <= 1) {
-            if (E < best1) {
-                best1 = E;
-                best1_x = x;
-            }
-            return;
-        }
-        if (codes.insert(x).second)
-            seen.emplace_back(E, x);
-    };
     std::mt19937_64 rng(0x9e3779b97f4a7c15ull ^ h.fix_value ^ ((uint64_t)n << 56));
-    std::vector<double> hf(n);
     for (int r = 0; r < restarts; ++r) {
         uint64_t x = base | (r == 0 ? 0 : (rng() & fmask));
-        double E = energy(x);
-        for (int j = 0; j < n; ++j) {
-            double a = 0.0;
-            for (int i = 0; i < n; ++i)
-                if (i != j && ((x >> i) & 1))
-                    a += U(i, j);
-            hf[j] = a;
+        double E = 0.0;
+        for (int j = 0; j < n; ++j)
+            g[j] = diag[j];
+        for (int i = 0; i < n; ++i) {
+            sgn[i] = ((x >> i) & 1) ? -1.0 : 1.0;
+            if (!((x >> i) & 1))
+                continue;
+            E += g[i];
+            for (int j = 0; j < n; ++j)
+                g[j] += S[i][j];
         }
         for (int it = 0; it < 4 * n + 8; ++it) {
             int best = -1;
             double bd = 0.0;
             for (int v = 0; v < free_bits; ++v) {
-                const double d = ((x >> v) & 1) ? -(U(v, v) + hf[v]) : (U(v, v) + hf[v]);
+                const double d = sgn[v] * g[v];
                 if (d < bd) {
                     bd = d;
                     best = v;
@@ -738,28 +732,59 @@ double threshold_bound(const HostInst &h, int K, int restarts)
             }
             if (best < 0)
                 break;
-            const bool up = !((x >> best) & 1);
+            const double sb = sgn[best];
             x ^= 1ull << best;
             E += bd;
             for (int j = 0; j < n; ++j)
-                if (j != best)
-                    hf[j] += up ? U(best, j) : -U(best, j);
+                g[j] += sb * S[best][j];
+            sgn[best] = -sb;
         }
-        // the local minimum and all its one-flip neighbours
-        offer(E, x);
+        // the local minimum and, for K > 1, all its one-flip neighbours (none of them lower)
+        if (K == 1) {
+            if (E < best1) {
+                best1 = E;
+                best1_x = x;
+            }
+            continue;
+        }
+        seen.emplace_back(E, x);
         for (int v = 0; v < free_bits; ++v)
-            offer(E + (((x >> v) & 1) ? -(U(v, v) + hf[v]) : (U(v, v) + hf[v])), x ^ (1ull << v));
+            seen.emplace_back(E + sgn[v] * g[v], x ^ (1ull << v));
     }
-    if (K <= 1 && restarts > 0)
-        seen.emplace_back(best1, best1_x);
-    K = std::max(K, 1);
-    if ((int)seen.size() < K)
-        return h.beta;
-    std::nth_element(seen.begin(), seen.begin() + (K - 1), seen.end());
-    double t = seen[K - 1].first;
+    double t;
+    uint64_t code;
+    if (K == 1) {
+        if (restarts <= 0)
+            return h.beta;
+        t = best1;
+        code = best1_x;
+    } else {
+        // the K-th lowest of the distinct states met
+        std::sort(seen.begin(), seen.end());
+        std::unordered_set<uint64_t> distinct;
+        size_t k = 0;
+        while (k < seen.size()) {
+            distinct.insert(seen[k].second);
+            if ((int)distinct.size() == K)
+                break;
+            ++k;
+        }
+        if (k >= seen.size())
+            return h.beta;
+        t = seen[k].first;
+        code = seen[k].second;
+    }
     if (h.is_float) {
         // the incremental energies above differ from the exact ones by rounding only
-        t = energy(seen[K - 1].second);
+        t = 0.0;
+        for (int i = 0; i < n; ++i) {
+            if (!((code >> i) & 1))
+                continue;
+            t += diag[i];
+            for (int j = i + 1; j < n; ++j)
+                if ((code >> j) & 1)
+                    t += S[i][j];
+        }
         t += 1e-9 * (1.0 + h.beta);
     } else {
         t = std::nearbyint(t);
