@@ -574,6 +574,7 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
         d.clampC = h.clampC;
         d.el_fused = j.acc == ACC_I16P && !grouped_form(j.acc, j.variant) ? h.el_fused : 0;
         d.elmin = h.elmin;
+        d.limb = j.acc == ACC_I64 && j.variant == kLimbVariant ? limb_shift(h) : 0;
         d.geps = 0.0f;
         if (j.acc == ACC_F32) {  // 16 ulp of beta: every column and E_L value is at most beta
             const float b = (float)h.beta;
@@ -1368,8 +1369,11 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order)
         if (tuned_plan(acc, 0, &tv, &tw))
             variant = tv;
     }
-    if (acc_bytes(acc) != 4)
-        variant = 0;
+    if (acc_bytes(acc) != 4) {
+        variant = acc == ACC_I64 ? kLimbVariant : 0;
+        for (auto &h : hs)
+            variant = limb_shift(h) > 0 ? variant : 0;
+    }
     const int wmax = batch_max_walk(acc, variant, hs, acc == ACC_F32 ? kFloatMaxWalkBits : kDefaultMaxWalkBits);
     int tuned[kMaxBatchedN + 1];
     batch_tuned_walks(acc, variant, tuned);
@@ -1509,6 +1513,7 @@ int prepare_folded(std::vector<int64_t> *Ui, std::vector<double> *Uf, int n, uin
     h = HostInst();
     h.n = n;
     h.is_float = Uf != nullptr;
+    h.plain = (flags & QUBO_FLAG_PLAIN) != 0;
     if (h.is_float) {
         h.Uf = std::move(*Uf);
         for (double v : h.Uf)
@@ -2464,6 +2469,7 @@ int qubo_autotune_batched_ex(const void *Q_packed, const int *n, const size_t *o
     const Acc acc = hs[0].acc;
     const bool lanes4 = acc_bytes(acc) == 4;
     const int nvar = lanes4 ? kScanVariants : 1;
+    const int variant8 = lanes4 ? 0 : hs[0].variant;  // the 8-byte accumulators' one variant of this batch
     // the untuned walk, as in batch_plan: as long as the instance allows, at most wmax (integers
     // in FP32 lanes: 2^14 steps when exact, else 2^12)
     const int wmax = acc == ACC_F32 ? kFloatMaxWalkBits : (acc == ACC_I32F ? kI32FMaxWalkBits : kDefaultMaxWalkBits);
@@ -2483,7 +2489,7 @@ int qubo_autotune_batched_ex(const void *Q_packed, const int *n, const size_t *o
     // not admitted (too short a walk, or lanes that would not stay exact).
     auto plan_one = [&](HostInst &h, int v, int w) -> bool {
         h.acc = acc;
-        h.variant = lanes4 ? v : 0;
+        h.variant = lanes4 ? v : variant8;
         const int B = acc_suffix_bits(acc, h.variant);
         const int rmin = reg_rows_of(acc, h.variant) + 1;
         const int wd = h.n - B >= rmin ? std::min(wmax, h.n - B) : 0;
@@ -2521,7 +2527,7 @@ int qubo_autotune_batched_ex(const void *Q_packed, const int *n, const size_t *o
             for (int i : order)
                 j.insts.push_back(&hv[i]);
             j.acc = acc;
-            j.variant = lanes4 ? v : 0;
+            j.variant = lanes4 ? v : variant8;
             j.margin = kDefaultMargin;
             std::vector<Part> parts;
             double gs = 0.0;
@@ -2608,6 +2614,8 @@ int qubo_autotune_batched_ex(const void *Q_packed, const int *n, const size_t *o
         }
         walk_of[nn] = wcur;
     }
+    if (!lanes4)
+        vbest = variant8;
     install_plan(acc, 0, vbest, 0);
     for (auto &kv : walk_of)
         install_plan(acc, -kv.first, vbest, kv.second);

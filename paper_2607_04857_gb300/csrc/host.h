@@ -72,6 +72,7 @@ struct HostInst {
     int32_t group_ok = 0;            // ACC_I16P: the plan can run a grouped variant (i16p_group_ok)
     int Z = 0;                  // ACC_I32Z / ACC_F32Z: walked rows without suffix couplings
     std::vector<uint8_t> perm;  // ACC_I32Z / ACC_F32Z: caller's variable at each scan position
+    bool plain = false;         // the plain form was asked for (QUBO_FLAG_PLAIN)
     bool no_factored = false;   // the factored FP32 scan used up its margin: plan the dense one
     int anchor_bits = kFloatAnchorBits;  // ACC_F32: re-anchoring period (log2 of walk steps)
     mutable Fp32BoundTerms fp32_terms;   // ACC_F32: cached magnitudes of the rounding bound
@@ -105,6 +106,7 @@ int reg_rows_of(Acc a, int variant);
 int variant_reg_rows(const HostInst &h);
 int scan_variant(Acc acc = ACC_I32);
 int pick_variant(Acc acc, int requested);
+int limb_shift(const HostInst &h);
 
 // The split n = k + L + B of a run (Sec. 3.3) and the accumulator it runs in: the exactness
 // checks of the packed 16-bit and FP32-lane scans, the factored scan's variable order.

@@ -70,11 +70,17 @@ constexpr int kPackedRegRows[kScanVariants] = {3, 3, 3, 3, 3, 2, 2, 2, 3, 3, 4, 
 constexpr int kPackedMinBlocks[kScanVariants] = {3, 3, 3, 4, 4, 2, 2, 4, 3, 4, 3, 4, 2, 2, 2, 2, 2, 1, 2, 2, 3, 3, 3, 4};
 constexpr int kPackedAddMode[kScanVariants] = {0, 3, 2, 0, 3, 0, 3, 3, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 3, 2, 0, 0, 0, 0};
 constexpr int kPackedInterleave[kScanVariants] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 0, 1, 1, 1, 1, 2, 2, 3, 3};
+// The 8-byte accumulators have variant 0; int64 also the grouped scan on two 32-bit limbs
+// (scan_i64.cu) for energies below 2^55, which keeps four register rows.
+constexpr int kLimbVariant = 1;
+constexpr int kLimbMaxShift = 26;
 // Whether a plan's scan kernel runs the grouped form.
 constexpr bool grouped_form(Acc acc, int variant)
 {
     if (variant < 0 || variant >= kScanVariants)
         return false;
+    if (acc == ACC_I64)
+        return variant == kLimbVariant;
     return acc == ACC_I16P ? kPackedInterleave[variant] == 2
                            : (acc == ACC_I32F || acc == ACC_F32 || acc == ACC_I32) && kVariantInterleave[variant] == 2;
 }
@@ -136,6 +142,7 @@ struct Inst {
                           // packed column minima without a carry (the host proves the sums fit 16 bits)
     int32_t elmin;        // ACC_I16P with el_fused: a lower bound of every E_L value
     float geps;           // ACC_F32, grouped form: rounding allowance of a group's column updates
+    int32_t limb;         // ACC_I64: > 0, energies on two limbs hi * 2^limb + lo (scan_i64.cu)
 };
 
 // Mutable per-instance state, updated with atomics.

@@ -98,6 +98,7 @@ int prepare(const void *Q, int n, qubo_dtype dt, uint32_t flags, HostInst &h)
             return QUBO_ERR_OVERFLOW;
         h.acc = ((flags & QUBO_FLAG_PLAIN) || beta >= (1ll << 30)) ? ACC_I64 : ACC_I32;
     }
+    h.plain = (flags & QUBO_FLAG_PLAIN) != 0;
     return QUBO_OK;
 }
 
@@ -127,7 +128,21 @@ int reg_rows_of(Acc a, int variant)
     const int v = variant >= 0 && variant < kScanVariants ? variant : 0;
     if (acc_factored(a))
         return 2;  // the factored scan needs at least 3 walked rows
-    return a == ACC_I16P ? kPackedRegRows[v] : kVariantRegRows[acc_bytes(a) == 4 ? v : 0];
+    if (acc_bytes(a) == 8)
+        return a == ACC_I64 && variant == kLimbVariant ? 4 : kVariantRegRows[0];
+    return a == ACC_I16P ? kPackedRegRows[v] : kVariantRegRows[v];
+}
+
+// Shift of the two-limb int64 scan, 0 when the plain kernel has to run: the limbs stay below 2^30 up
+// to beta < 2^55, and the plain form is what QUBO_FLAG_PLAIN asks for.
+int limb_shift(const HostInst &h)
+{
+    if (h.is_float || h.plain || !(h.beta < 36028797018963968.0))
+        return 0;
+    int s = 1;
+    while (std::ldexp(1.0, 29 + s) < h.beta)
+        ++s;
+    return s;
 }
 
 // Walked rows the run's kernel variant keeps in registers (a walk needs at least one more bit).
@@ -676,9 +691,16 @@ int plan_run(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int wal
         }
         h.acc = chosen;
     }
-    h.variant = acc_bytes(h.acc) == 4 ? pick_variant(h.acc, variant_req) : 0;
-    if (acc_bytes(h.acc) == 4)
+    if (acc_bytes(h.acc) == 4) {
+        h.variant = pick_variant(h.acc, variant_req);
         h.variant = fit_variant(h, fix_bits, split_k, walk_bits, variant_req, h.variant);
+    } else {
+        // the two-limb kernel where its walk (at least five bits) fits
+        const int bits = h.n - fix_bits - acc_suffix_bits(h.acc, 0);
+        const int L = split_k > 0 ? h.n - acc_suffix_bits(h.acc, 0) - split_k : walk_bits > 0 ? walk_bits : bits;
+        h.variant = h.acc == ACC_I64 && L >= 5 && L <= (split_k > 0 || walk_bits > 0 ? kGroupedMaxWalkBits : L) &&
+                            limb_shift(h) > 0 ? kLimbVariant : 0;
+    }
     if (h.acc == ACC_I16P)
         h.variant = packed_variant_for(h.variant, h.group_ok, h.el_fused);
     return plan(h, fix_bits, fix_value, split_k, walk_bits);

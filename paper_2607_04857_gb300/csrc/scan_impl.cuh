@@ -75,7 +75,7 @@ struct Tr<int32_t> {
 
 template <>
 struct Tr<int64_t> {
-    static constexpr bool kGrouped = false;
+    static constexpr bool kGrouped = true;  // the two-limb kernel (scan_i64.cu)
     using TC = int64_t;
     using TP = int64_t;
     static constexpr bool kIntInFloat = false;
@@ -399,7 +399,12 @@ __global__ void tables_kernel(const Inst *insts)
                 ((TC *)d.Es)[j] = (TC)acc;
         } else if (idx < NB + NM * L) {
             const long r = (idx - NB) / NM, w = (idx - NB) % NM;
-            if constexpr (kPacked)  // packed delta: column w in the low lane, w + NB/2 in the high
+            if (std::is_same_v<T, int64_t> && d.limb) {  // two limbs: the row's hi values, then its lo values
+                const int64_t v = (int64_t)m_entry(r, w);
+                const int64_t lo = (int64_t)((uint64_t)v << (64 - d.limb)) >> (64 - d.limb);
+                ((int32_t *)d.M)[r * 2 * NM + w] = (int32_t)((v - lo) >> d.limb);
+                ((int32_t *)d.M)[r * 2 * NM + NM + w] = (int32_t)lo;
+            } else if constexpr (kPacked)  // packed delta: column w in the low lane, w + NB/2 in the high
                 ((TC *)d.M)[r * NM + w] = (uint32_t)m_entry(r, w) + ((uint32_t)m_entry(r, w + NB / 2) << 16);
             else
                 ((TC *)d.M)[r * NM + w] = (TC)m_entry(r, w);

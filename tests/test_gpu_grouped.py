@@ -196,3 +196,47 @@ def test_float_proven_margin_gives_up(q):
     o = oracle.solve(Q, topk=4096, cap=1)
     sel = o.topk_E <= o.min + 2e-4
     assert not sel.all() and cnt == int(sel.sum()) and np.array_equal(codes, o.topk[sel])
+
+
+# --- int64 energies on two limbs -----------------------------------------------------------------
+
+@pytest.mark.parametrize("walk", [0, 5, 6, 9, 14])
+@pytest.mark.parametrize("scale", [1 << 22, 1 << 26, (1 << 31) - 1])
+def test_two_limbs(q, walk, scale):
+    """Energies from just beyond int32 to the largest an int32 matrix gives, on random entries and on
+    entries whose low halves all lie at the split's extremes."""
+    n = 25
+    Q = wl.upper_int(n, -scale, scale, seed=walk + 3).astype(np.int64)
+    iu = np.triu_indices(n)
+    for low in (None, 0x2aaaaa, -1):
+        M = Q.copy()
+        if low is not None:
+            M[iu] = (M[iu] >> 23 << 23) + (low & 0x3fffff) if scale > 1 << 24 else M[iu] | 1
+        M = np.clip(M, -(2**31), 2**31 - 1).astype(np.int32)
+        M[0, 0] = 2**31 - 1  # the sum of |U| above 2^30
+        r, o = q.solve(M, topk=9, walk_bits=walk), oracle.solve(M, topk=9)
+        assert r.info["acc"] == "i64" and r.info["grouped"] == 1, r.info
+        check(r, o)
+        check(q.solve(M, walk_bits=walk), oracle.solve(M))
+    p = q.solve(M, topk=9, plain=True)
+    assert p.info["acc"] == "i64" and p.info["grouped"] == 0
+    check(p, oracle.solve(M, topk=9))
+
+
+def test_two_limbs_ties_window_batch(q):
+    """Ties in every group, every state of a window, and a batch with direct evaluation beside it."""
+    Q = np.zeros((24, 24), dtype=np.int32)
+    Q[np.arange(10), np.arange(10)] = -(1 << 30)
+    check(q.solve(Q, states_cap=1 << 14), oracle.solve(Q, cap=1 << 14))
+    W = wl.upper_int(24, -(1 << 27), 1 << 27, seed=8)
+    o = oracle.solve(W, topk=4096, cap=1)
+    width = int(o.topk_E[900] - o.min)
+    sel = o.topk_E <= o.min + width
+    if width < 1 << 30:
+        cnt, codes, E, info = q.solve_window(W, width)
+        assert info["acc"] == "i64" and cnt == int(sel.sum())
+        assert np.array_equal(codes, o.topk[sel]) and np.array_equal(E, o.topk_E[sel])
+    insts = [wl.upper_int(n, -(1 << 28), 1 << 28, seed=n) for n in (9, 13, 14, 15, 19, 22)]
+    for M, r in zip(insts, q.solve_batched(insts, topk=4)):
+        assert r.info["acc"] == "i64"
+        check(r, oracle.solve(M, topk=4, cap=64))
