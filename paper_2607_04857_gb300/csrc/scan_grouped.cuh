@@ -1,21 +1,19 @@
 // The grouped step form of the dense scans (included by scan_impl.cuh, which has its helpers).
 //
 // The min over a step's columns is half of a state's work and only finds the rare states at or
-// below the threshold.  The walk runs in groups of 16 Gray steps.  At a group's first state each
-// thread takes the exact minimum m of its columns.  Steps 1..15 of a group flip the register rows
-// 0-3, in the same pattern in every group but for the sign of row 3, which alternates, and a flip
-// moves column q by +-M_r[q]; so over the group the thread's minimum never falls below m + D, D the
-// smallest running sum of the steps' smallest column moves (min_q M_r[q] on an add, -max_q M_r[q]
-// on a subtract; two values per thread and unit, one per sign of row 3).  With min E_L over the
+// below the threshold.  The walk runs in groups of 16 Gray steps.  Steps 1..15 of a group flip the
+// register rows 0-3, in the same pattern in every group but for the sign of row 3, which alternates:
+// the group's 16 states of a column are its value with rows 0-3 clear plus every subset of the four
+// rows, so its minimum over the group is its value at the first state plus an offset, the sum of the
+// rows' negative parts, less M_3 when row 3 is set there.  At a group's first state each thread takes
+// the exact minimum m of its columns; with D the smallest offset of its columns (two values per thread
+// and unit, one per sign of row 3), no column falls below m + D in the group.  With min E_L over the
 // group's states from the tables, m + D > u - min E_L in every lane proves that the group holds no
-// candidate, and it runs its 15 column updates alone; otherwise it takes the column minima step by
-// step and a hit rebuilds the group's states.  Every state gets its column update either way.
+// candidate, and it runs its 15 column updates alone.  Every state gets its column update either way.
 //
-// A group the first test cannot clear takes a second, exact one.  Within a group the 16 states of a
-// column are its value with rows 0-3 clear plus every subset of the four rows, so its minimum over
-// the group is that value plus the sum of the rows' negative parts (kept per column in shared
-// memory); the smallest of these over the columns, plus min E_L, bounds the group from below with
-// no slack but E_L's.
+// A group the first test cannot clear takes a second one, each column with its own offset (kept in
+// shared memory): the exact minimum over the group, with no slack but E_L's.  Groups that fail it
+// (n=36: 0.002% of them, n=48 Max-Cut 0.004%) are walked state by state.
 //
 // What bounds it (GB300, cycles per 16-column step per scheduler): eight f32x2 adds 16.1 (both halves
 // of the FMA pipe); sixteen int32 adds 16 when half of them issue to the FMA pipe's heavy half and
@@ -104,23 +102,6 @@ __device__ __forceinline__ float add_down(float a, float b) { return __fadd_rd(a
 __device__ __forceinline__ int32_t add_down(int32_t a, int32_t b) { return a + b; }
 __device__ __forceinline__ int64_t add_down(int64_t a, int64_t b) { return a + b; }
 
-// D for each sign of row 3 (PAR) from the smallest and largest move of rows 0-3.
-template <class DD>
-__device__ __forceinline__ void group_bounds(const DD (&lo)[4], const DD (&hi)[4], DD (&D)[2])
-{
-    static_for<2>([&](auto pc) {
-        constexpr int par = decltype(pc)::value;
-        DD cum = 0, least = 0;
-        static_for<15>([&](auto tc) {
-            constexpr int t = decltype(tc)::value + 1, kk = ctzc(t);
-            constexpr bool neg = kk == 3 ? par != 0 : ((t >> (kk + 1)) & 1) != 0;
-            cum += neg ? -hi[kk] : lo[kk];
-            least = min(least, cum);
-        });
-        D[par] = least;
-    });
-}
-
 // One work unit of the grouped form: all 2^(B+L) states with fixed bits x_f = unit, L >= 5.
 // FP32 columns that hold integers: m + D is summed rounding down and u - min E_L is exact (both
 // stay below 2^24).  FP32 columns of float Q take 16 ulp of beta (geps) off m + D, more than the
@@ -197,47 +178,29 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
         }
     }
 
-    // the negative parts of rows 0-3 per column, summed rounding down
-    __syncwarp();
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        TC nv[V];
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-            nv[e] = emin(Mr[0][g * V + e], (TC)0);
-#pragma unroll
-            for (int r = 1; r < 4; ++r)
-                nv[e] = add_down(nv[e], emin(Mr[r][g * V + e], (TC)0));
-        }
-        *(typename VecOf<TC>::type *)(neg + (g * 32 + lane) * V) = vjoin(nv);
-    }
-
-    using DD = std::conditional_t<Tr<T>::kFloat, double, int64_t>;
+    // the offsets (rows 0-3 clear at the first state) and D, summed rounding down
     using DB = std::conditional_t<kFp, float, int64_t>;  // the bound as the test takes it
     DB Dgrp[2];
     {
-        DD lo4[4], hi4[4], D[2];
+        TC d0{}, d1{};
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            TC lo = Mr[r][0], hi = Mr[r][0];
+        for (int g = 0; g < G; ++g) {
+            TC nv[V];
 #pragma unroll
-            for (int q = 1; q < S; ++q) {
-                lo = emin(lo, Mr[r][q]);
-                hi = hi > Mr[r][q] ? hi : Mr[r][q];
+            for (int e = 0; e < V; ++e) {
+                const int q = g * V + e;
+                nv[e] = emin(Mr[0][q], (TC)0);
+#pragma unroll
+                for (int r = 1; r < 4; ++r)
+                    nv[e] = add_down(nv[e], emin(Mr[r][q], (TC)0));
+                const TC odd = add_down(nv[e], -Mr[3][q]);
+                d0 = q ? emin(d0, nv[e]) : nv[e];
+                d1 = q ? emin(d1, odd) : odd;
             }
-            lo4[r] = (DD)lo;
-            hi4[r] = (DD)hi;
+            *(typename VecOf<TC>::type *)(neg + (g * 32 + lane) * V) = vjoin(nv);
         }
-        group_bounds(lo4, hi4, D);
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            if constexpr (Tr<T>::kFloat)
-                Dgrp[p] = __double2float_rd(D[p]);
-            else if constexpr (kFp)
-                Dgrp[p] = __ll2float_rd(D[p]);
-            else
-                Dgrp[p] = D[p];
-        }
+        Dgrp[0] = (DB)d0;
+        Dgrp[1] = (DB)d1;
     }
     keep_mad_rows(Mr, a.mad_inverse);
 
@@ -567,7 +530,7 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
 
 // One work unit of the grouped form in packed 16-bit columns (see scan_unit_packed for the lanes).
 // E_L is stored minus the lane bias, so lane + stored E_L is the column's energy without P.  D takes
-// the moves of both lanes; the host admits only plans whose rows 0-3 move a column by at most 32767.
+// the offsets of both lanes; the host admits only plans whose rows 0-3 move a column by at most 32767.
 template <int S, int RC, int NG, bool K1>
 __device__ __forceinline__ void scan_unit_packed_grouped(const ScanArgs &a, const Inst &d, int inst, uint64_t unit,
                                                          int32_t &Treg, int lane, uint32_t *stage, int32_t *wsm,
@@ -621,33 +584,28 @@ __device__ __forceinline__ void scan_unit_packed_grouped(const ScanArgs &a, cons
                 Mr[r][g * V + e] = mv[e] + wr2;
         }
     }
-    // D, and the negative parts of rows 0-3 per lane; a row's word is x + 65536 y with both moves in
+    // the offsets per lane and D over both lanes; a row's word is x + 65536 y with both moves in
     // [-32768, 32767]
-    int32_t Dgrp[2];
-    {
-        int32_t lo4[4] = {0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff};
-        int32_t hi4[4] = {-0x7fffffff, -0x7fffffff, -0x7fffffff, -0x7fffffff};
-        __syncwarp();
+    int32_t Dgrp[2] = {0x7fffffff, 0x7fffffff};
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            uint32_t nv[V];
+    for (int g = 0; g < G; ++g) {
+        uint32_t nv[V];
 #pragma unroll
-            for (int e = 0; e < V; ++e) {
-                int32_t nx = 0, ny = 0;
+        for (int e = 0; e < V; ++e) {
+            int32_t nx = 0, ny = 0, x = 0, y = 0;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint32_t w = Mr[r][g * V + e];
-                    const int32_t x = (int32_t)(int16_t)(w & 0xffffu), y = (int32_t)(w - (uint32_t)x) >> 16;
-                    lo4[r] = __vimin3_s32(lo4[r], x, y);
-                    hi4[r] = __vimax3_s32(hi4[r], x, y);
-                    nx += min(x, 0);
-                    ny += min(y, 0);
-                }
-                nv[e] = (uint32_t)nx + ((uint32_t)ny << 16);
+            for (int r = 0; r < 4; ++r) {
+                const uint32_t w = Mr[r][g * V + e];
+                x = (int32_t)(int16_t)(w & 0xffffu);
+                y = (int32_t)(w - (uint32_t)x) >> 16;
+                nx += min(x, 0);
+                ny += min(y, 0);
             }
-            *(uint4 *)(neg + (g * 32 + lane) * V) = vjoin(nv);
+            nv[e] = (uint32_t)nx + ((uint32_t)ny << 16);
+            Dgrp[0] = __vimin3_s32(Dgrp[0], nx, ny);
+            Dgrp[1] = __vimin3_s32(Dgrp[1], nx - x, ny - y);
         }
-        group_bounds(lo4, hi4, Dgrp);
+        *(uint4 *)(neg + (g * 32 + lane) * V) = vjoin(nv);
     }
     keep_mad_rows(Mr, a.mad_inverse);
 

@@ -76,29 +76,21 @@ __device__ __forceinline__ void scan_unit_limbs(const ScanArgs &a, const Inst &d
     }
     int64_t Dgrp[2];
     {
-        int64_t lo4[4], hi4[4];
+        int32_t d0 = 0x7fffffff, d1 = 0x7fffffff;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            int32_t lo = Mh[r][0], hi = Mh[r][0];
+        for (int g = 0; g < G; ++g) {
+            int32_t nv[V];
 #pragma unroll
-            for (int q = 1; q < S; ++q) {
-                lo = min(lo, Mh[r][q]);
-                hi = max(hi, Mh[r][q]);
+            for (int e = 0; e < V; ++e) {
+                const int q = g * V + e;
+                nv[e] = min(Mh[0][q], 0) + min(Mh[1][q], 0) + min(Mh[2][q], 0) + min(Mh[3][q], 0);
+                d0 = min(d0, nv[e]);
+                d1 = min(d1, nv[e] - Mh[3][q]);
             }
-            lo4[r] = lo;
-            hi4[r] = hi;
+            *(int4 *)(sm.neg + (g * 32 + lane) * V) = vjoin(nv);
         }
-        group_bounds(lo4, hi4, Dgrp);
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        int32_t nv[V];
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-            const int q = g * V + e;
-            nv[e] = min(Mh[0][q], 0) + min(Mh[1][q], 0) + min(Mh[2][q], 0) + min(Mh[3][q], 0);
-        }
-        *(int4 *)(sm.neg + (g * 32 + lane) * V) = vjoin(nv);
+        Dgrp[0] = d0;
+        Dgrp[1] = d1;
     }
     keep_mad_rows(Mh, a.mad_inverse);
     keep_mad_rows(Ml, a.mad_inverse);

@@ -109,3 +109,19 @@ def test_exact_group_minimum(seed):
             col = col + (-1 if neg else 1) * rows[kk]
             least = np.minimum(least, col)
         assert np.array_equal(least, first - par * rows[3] + np.minimum(rows, 0).sum(axis=0))
+
+
+@pytest.mark.parametrize("seed", range(3))
+def test_smallest_offset_bounds_every_column(seed):
+    """The first test's bound: m + D, D the smallest over a thread's columns of the offset between a
+    column's group minimum and its value at the group's first state, is at or below every column in the
+    group and at least as tight as the running sums of extreme moves."""
+    rng = np.random.default_rng(100 + seed)
+    rows, start = rng.integers(-80, 81, size=(4, 16)), rng.integers(-400, 400, size=16)
+    neg = np.minimum(rows, 0).sum(axis=0)
+    for par in (0, 1):
+        first = start + par * rows[3]
+        D = (neg - par * rows[3]).min()
+        least = min((start + sum(((p >> r) & 1) * rows[r] for r in range(4))).min() for p in range(16))
+        assert first.min() + D <= least
+        assert D >= group_bound(rows, np.zeros(4, dtype=np.int64), par)
