@@ -1170,17 +1170,17 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
     int st;
     const bool fp32 = h.acc == ACC_F32 && !(c.flags & (QUBO_FLAG_PLAIN | QUBO_FLAG_RIGOROUS));
     bool done = false, tried = false;
-    if (fp32 && !(float_slack(h) < c.margin)) {  // no drift, however small, would fit the margin
+    if (fp32 && !(2.0 * float_slack(h) < c.margin)) {  // little or no room for a drift in the margin
         tried = true;
         if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
             return st;
         if (!done && !h.small)
-            h.acc = ACC_F64;
+            h.acc = float_slack(h) < c.margin ? ACC_F32 : ACC_F64;
     }
     if (!done && (st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))
         return st;
-    // FP32 drift above the margin's budget: shorten the re-anchoring period, then take a proven
-    // margin, and as a last resort rescan in FP64.
+    // FP32 drift above the margin's budget: take a proven margin with a shorter re-anchoring period; when
+    // that gives up, shorten the period further, and as a last resort rescan in FP64.
     while (!done && !float_margin_ok(h, p, c.margin)) {
         const int period = std::min(h.anchor_bits, h.L);
         if (h.acc == ACC_F32Z) {  // the dense FP32 scan next
@@ -1189,14 +1189,15 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
             c.walk_bits = o.walk_bits;
         } else if (h.acc == ACC_F32 && !h.small && period > variant_reg_rows(h) + 1) {
             h.anchor_bits = std::max(variant_reg_rows(h) + 1, period - 2);
-        } else {
             if (fp32 && !tried) {
                 tried = true;
                 if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
                     return st;
                 if (done)
                     break;
+                h.acc = ACC_F32;
             }
+        } else {
             h.acc = ACC_F64;
             c.walk_bits = o.walk_bits;
         }

@@ -291,8 +291,8 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
     const TC *ELg = ELp + (1 << L);  // min E_L over each group
     const uint64_t cbase = unit << BL;
 
-    // The group of 16 states whose first is in E: the tests, then the column updates; true when a
-    // column of this thread may be at or below the threshold in one of its states.  PAR: sign of row
+    // The group of 16 states whose first is in E: the tests, then the column updates; true (for
+    // the warp) when a column may be at or below the threshold in one of its states.  PAR: sign of row
     // 3 (2: par, at run time).
     auto run_group = [&](auto parc, int par, TC elg) -> bool {
         constexpr int PAR = decltype(parc)::value;
@@ -339,35 +339,29 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
                 updates();
                 return false;
             }
-            const bool hit = !above(refined());
+            const bool hit = !__all_sync(kFull, above(refined()));
             updates();
             return hit;
         } else {
             bool hit = false;
             if (!clear)
-                hit = !above(refined());
+                hit = !__all_sync(kFull, above(refined()));
             updates();
             return hit;
         }
     };
 
-    // Rare: offer the staged columns of walk step i (P = Pp, E_L = elp) at or below the threshold tp.
-    auto record_staged = [&](int i, TP Pp, TC elp, TC tp) {
+    // Rare: offer the staged columns in mask of walk step i (P = Pp, E_L = elp).
+    auto record_staged = [&](int i, TP Pp, TC elp, unsigned mask) {
         const uint64_t cb = cbase | ((uint64_t)(i ^ (i >> 1)) << B);
         const TP Ep = Pp + (TP)elp;
-#pragma unroll 1
-        for (int q = 0; q < S; ++q) {
-            const TC v = stage[q * 32 + lane];
-            if (v <= tp) {
-                const TP Et = (TP)v + Ep;
-                const uint32_t j = (uint32_t)(((q / V) * 32 + lane) * V + (q % V));
-                record<T>(a, inst, Et, cb | j);
-                if (K1 && Et < Treg) {
-                    Treg = Et;
-                    tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
-                    Tr<T>::thr_min(st, Et);
-                }
-            }
+        const TP least = record_warp<T>(
+            a, inst, mask, lane, [&](int q) { return (TP)stage[q * 32 + lane] + Ep; },
+            [&](int q) { return cb | (uint32_t)(((q / V) * 32 + lane) * V + (q % V)); });
+        if (K1 && least < Treg) {
+            Treg = least;
+            if (lane == 0)
+                Tr<T>::thr_min(st, least);
         }
     };
     // Columns of walk step i of the body from those of step j: the register rows, and with NG > 1 row
@@ -395,7 +389,7 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
             });
         });
     };
-    // The states of the body's groups in hits, E being the body's last one.  Integer columns (exact)
+    // The states of the body's groups in hits (the same for the warp), E being the body's last one.  Integer columns (exact)
     // are moved to each group's first state, walked through it and moved back; FP32 columns are
     // left alone and every state is rebuilt from the last one.  Pmid: P before the flip of row RC.
     auto record_hits = [&](int i0, unsigned hits, TP Pmid) {
@@ -409,16 +403,16 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
             for (int p = 0; p < BODY; ++p) {
                 if (!((hits >> (p >> 4)) & 1u))
                     continue;
-                if (gave_up(a))
+                if (__any_sync(kFull, gave_up(a)))
                     break;
                 const int i = i0 + p, gp = i ^ (i >> 1);
-                TC sr[NR], least{};
+                TC sr[NR];
 #pragma unroll
                 for (int r = 0; r < NR; ++r)
                     sr[r] = (TC)(((gp >> r) & 1) - ((gend >> r) & 1));
                 const TP Pp = prefix(i);
-                const TC elp = ELp[i];
-                TC tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
+                const TC elp = ELp[i], tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
+                unsigned mask = 0;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
                     TC mv[V];
@@ -434,11 +428,11 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
                         if constexpr (NG > 1)
                             x = x + sr[RC] * mv[e];
                         stage[q * 32 + lane] = x;
-                        least = q == 0 ? x : emin(least, x);
+                        mask |= x <= tp ? 1u << q : 0u;
                     }
                 }
-                if (least <= tp)
-                    record_staged(i, Pp, elp, tp);
+                if (__any_sync(kFull, mask != 0))
+                    record_staged(i, Pp, elp, mask);
             }
         } else {
             int at = iend;
@@ -463,12 +457,15 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
                 at = i0 + p;
                 const TP Pp = prefix(at);
                 const TC elp = ELp[at], tp = to_col<T>(Treg + mu - Pp, clampC) - elp;
-                if (!(tree_min<TC, 3, S>(E) <= tp))
+                if (!__any_sync(kFull, tree_min<TC, 3, S>(E) <= tp))
                     continue;
+                unsigned mask = 0;
 #pragma unroll
-                for (int q = 0; q < S; ++q)
+                for (int q = 0; q < S; ++q) {
                     stage[q * 32 + lane] = E[q];
-                record_staged(at, Pp, elp, tp);
+                    mask |= E[q] <= tp ? 1u << q : 0u;
+                }
+                record_staged(at, Pp, elp, mask);
             }
             move(E, iend, at);
         }
@@ -656,7 +653,7 @@ __device__ __forceinline__ void scan_unit_packed_grouped(const ScanArgs &a, cons
                     low[q] = (odd ? E[q] - mad_factor<uint32_t>(3, q) * Mr[3][q] : E[q]) + nv[e];
                 }
             }
-            hit = lane_min(tree_min<uint32_t, 3, S>(low)) <= u - elg;
+            hit = !__all_sync(kFull, lane_min(tree_min<uint32_t, 3, S>(low)) > u - elg);
         }
         if constexpr (PAR == 2) {
             if (odd)
@@ -671,29 +668,31 @@ __device__ __forceinline__ void scan_unit_packed_grouped(const ScanArgs &a, cons
 
     constexpr int LOGBODY = 4 + ilog2c(NG), BODY = 1 << LOGBODY;
     auto record_state = [&](int i, int32_t Pp) {
-        const int32_t els = ELp[i];
-        int32_t tp = Treg + mu - Pp - els;
-        if (lane_min(tree_min<uint32_t, 3, S>(E)) > tp)
+        const int32_t els = ELp[i], tp = Treg + mu - Pp - els;
+        if (!__any_sync(kFull, lane_min(tree_min<uint32_t, 3, S>(E)) <= tp))
             return;
+        unsigned mask = 0;  // bit 2 q + h: half h of word q
 #pragma unroll
-        for (int q = 0; q < S; ++q)
+        for (int q = 0; q < S; ++q) {
             stage[q * 32 + lane] = E[q];
+            mask |= (int32_t)(E[q] & 0xffffu) <= tp ? 1u << (2 * q) : 0u;
+            mask |= (int32_t)(E[q] >> 16) <= tp ? 2u << (2 * q) : 0u;
+        }
         const uint64_t cb = cbase | ((uint64_t)(i ^ (i >> 1)) << B);
-#pragma unroll 1
-        for (int q = 0; q < 2 * S; ++q) {
-            const int qw = q >> 1;
-            const uint32_t word = stage[qw * 32 + lane];
-            const int32_t x = (int32_t)((q & 1) ? (word >> 16) : (word & 0xffffu));
-            if (x <= tp) {
-                const int32_t Et = x + els + Pp;
-                const uint32_t j = (uint32_t)(((qw / V) * 32 + lane) * V + (qw % V)) + ((q & 1) ? NW : 0);
-                record<T>(a, inst, Et, cb | j);
-                if (K1 && Et < Treg) {
-                    Treg = Et;
-                    tp = Treg + mu - Pp - els;
-                    Tr<T>::thr_min(st, Et);
-                }
-            }
+        const int32_t least = record_warp<T>(
+            a, inst, mask, lane,
+            [&](int q) {
+                const uint32_t word = stage[(q >> 1) * 32 + lane];
+                return (int32_t)((q & 1) ? (word >> 16) : (word & 0xffffu)) + els + Pp;
+            },
+            [&](int q) {
+                const int w = q >> 1;
+                return cb | (uint32_t)(((w / V) * 32 + lane) * V + (w % V) + ((q & 1) ? NW : 0));
+            });
+        if (K1 && least < Treg) {
+            Treg = least;
+            if (lane == 0)
+                Tr<T>::thr_min(st, least);
         }
     };
     const uint32_t *rowRC = Mt + (size_t)RC * NW;

@@ -124,28 +124,27 @@ __device__ __forceinline__ void scan_unit_limbs(const ScanArgs &a, const Inst &d
                 });
             }
             const int i = i0 + t;
-            const int64_t el = ELp[i];
-            int64_t tp = u - el;
-            if ((int64_t)tree_min<int32_t, 3, S>(Eh) > (tp >> s) + 8)
+            const int64_t el = ELp[i], tp = u - el;
+            if (!__any_sync(kFull, (int64_t)tree_min<int32_t, 3, S>(Eh) <= (tp >> s) + 8))
                 continue;
+            unsigned mask = 0;
 #pragma unroll
-            for (int q = 0; q < S; ++q)
-                sm.stage[q * 32 + lane] = (int64_t)Eh[q] * ((int64_t)1 << s) + El[q];
-            const uint64_t cb = cbase | ((uint64_t)(i ^ (i >> 1)) << B);
-#pragma unroll 1
             for (int q = 0; q < S; ++q) {
-                const int64_t x = sm.stage[q * 32 + lane];
-                if (x <= tp) {
-                    const int64_t Et = x + el + P;
-                    const uint32_t j = (uint32_t)(((q / V) * 32 + lane) * V + (q % V));
-                    record<T>(a, inst, Et, cb | j);
-                    if (K1 && Et < Treg) {
-                        Treg = Et;
-                        u = Treg + mu - P;
-                        tp = u - el;
-                        Tr<T>::thr_min(st, Et);
-                    }
-                }
+                const int64_t x = (int64_t)Eh[q] * ((int64_t)1 << s) + El[q];
+                sm.stage[q * 32 + lane] = x;
+                mask |= x <= tp ? 1u << q : 0u;
+            }
+            if (!__any_sync(kFull, mask != 0))
+                continue;
+            const uint64_t cb = cbase | ((uint64_t)(i ^ (i >> 1)) << B);
+            const int64_t least = record_warp<T>(
+                a, inst, mask, lane, [&](int q) { return sm.stage[q * 32 + lane] + el + P; },
+                [&](int q) { return cb | (uint32_t)(((q / V) * 32 + lane) * V + (q % V)); });
+            if (K1 && least < Treg) {
+                Treg = least;
+                u = Treg + mu - P;
+                if (lane == 0)
+                    Tr<T>::thr_min(st, least);
             }
         }
     };

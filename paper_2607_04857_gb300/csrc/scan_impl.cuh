@@ -355,6 +355,56 @@ __device__ __forceinline__ void record(const ScanArgs &a, int inst, typename Tr<
     Tr<T>::gmin_min(st, E);
 }
 
+// Offer the states in a warp's masks (bit q of lane l: the state with energy energy(q) and code code(q)
+// there) to the candidate buffer: one pair of atomics for all of them, whose latency a state-by-state
+// record pays each time.  Every lane takes part.  Returns the smallest energy offered.
+template <class T, class EnergyFn, class CodeFn>
+__device__ __forceinline__ typename Tr<T>::TP record_warp(const ScanArgs &a, int inst, unsigned mask, int lane,
+                                                          EnergyFn &&energy, CodeFn &&code)
+{
+    using TP = typename Tr<T>::TP;
+    InstState *st = a.state + inst;
+    const int cnt = __popc(mask);
+    int upto = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, upto, o);
+        if (lane >= o)
+            upto += v;
+    }
+    const unsigned long long total = (unsigned)__shfl_sync(kFull, upto, 31);
+    unsigned long long base = 0;
+    if (lane == 0) {
+        base = atomicAdd(a.nrec, total);
+        atomicAdd(&st->nrec, total);
+        if (base + total > a.rec_cap)
+            atomicAdd(&st->dropped, base >= a.rec_cap ? total : base + total - a.rec_cap);
+    }
+    base = __shfl_sync(kFull, base, 0);
+    unsigned long long idx = base + (unsigned)(upto - cnt);
+    TP least = std::is_same_v<TP, float> ? (TP)__int_as_float(0x7f800000)
+               : sizeof(TP) == 4         ? (TP)0x7fffffff
+                                         : (TP)0x7fffffffffffffffll;
+    for (; mask; mask &= mask - 1, ++idx) {
+        const int q = __ffs(mask) - 1;
+        const TP E = energy(q);
+        least = emin(least, E);
+        if (idx < a.rec_cap) {
+            Rec r;
+            r.key = a.n_inst > 1 ? (((uint64_t)inst << kInstShift) | code(q)) : code(q);
+            r.e = Tr<T>::bits(E);
+            a.rec[idx] = r;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        least = emin(least, (TP)__shfl_xor_sync(kFull, least, o));
+    if (lane == 0 && total)
+        Tr<T>::gmin_min(st, least);
+    return least;
+}
+
 // ---- table build (preprocessing of Alg. 1-2: E(U_B), M_int = Q_ps U_B^T, E(U_A)) ------------------
 // One thread per table entry; entries are subset sums of the symmetric coupling matrix W.
 template <class T>
