@@ -574,6 +574,8 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
         d.clampC = h.clampC;
         d.el_fused = j.acc == ACC_I16P && !grouped_form(j.acc, j.variant) ? h.el_fused : 0;
         d.elmin = h.elmin;
+        for (int r = 0; r < 4; ++r)
+            d.center[r] = grouped_form(j.acc, j.variant) ? h.center[r] : 0;
         d.limb = j.acc == ACC_I64 && j.variant == kLimbVariant ? limb_shift(h) : 0;
         d.geps = 0.0f;
         if (j.acc == ACC_F32) {  // 16 ulp of beta: every column and E_L value is at most beta
@@ -1450,6 +1452,10 @@ int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order)
         for (int i = 0; i < count; ++i)
             set_plan_fields(hs[i], saved[i]);
     }
+    parallel([&](int lo, int hi) {
+        for (int i = lo; i < hi; ++i)
+            center_rows(hs[i]);
+    });
     // longest work first (LPT order) so the tail of the persistent launch is short
     order.resize(count);
     for (int i = 0; i < count; ++i)
@@ -2514,11 +2520,16 @@ int qubo_autotune_batched_ex(const void *Q_packed, const int *n, const size_t *o
                 return i32f_exact(h, &h.clampC);
             return true;
         };
+        auto centered = [&](bool ok) {
+            if (ok)
+                center_rows(h);
+            return ok;
+        };
         if (w > 0)
-            return admitted(w);
+            return centered(admitted(w));
         if (admitted(wd))
-            return true;
-        return acc == ACC_I32F && wd > kDefaultMaxWalkBits && admitted(kDefaultMaxWalkBits);
+            return centered(true);
+        return centered(acc == ACC_I32F && wd > kDefaultMaxWalkBits && admitted(kDefaultMaxWalkBits));
     };
     // Device time (tables, scan, reduction) of one launch over the whole batch, best of two.
     auto time_batch = [&](std::vector<HostInst> &hv, int v, double *t) -> int {

@@ -69,6 +69,8 @@ struct HostInst {
     int32_t clampC = 0; // ACC_I32F: threshold clamp
     int32_t col_lo = 0, col_hi = 0;  // ACC_I16P: proven range of every column value
     int32_t el_fused = 0, elmin = 0; // ACC_I16P: E_L added to the packed minima (i16p_fuse_el)
+    int32_t center[4] = {0, 0, 0, 0};  // grouped integer scans: center_rows
+    double i32f_room = 0.0;          // ACC_I32F: what its values may grow by and stay exact
     int32_t group_ok = 0;            // ACC_I16P: the plan can run a grouped variant (i16p_group_ok)
     int Z = 0;                  // ACC_I32Z / ACC_F32Z: walked rows without suffix couplings
     std::vector<uint8_t> perm;  // ACC_I32Z / ACC_F32Z: caller's variable at each scan position
@@ -112,12 +114,13 @@ int limb_shift(const HostInst &h);
 // checks of the packed 16-bit and FP32-lane scans, the factored scan's variable order.
 int grouped_walk(int bits, int lmin, int lmax);
 int plan(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bits);
-bool i32f_exact(const HostInst &h, int32_t *clampC);
+bool i32f_exact(HostInst &h, int32_t *clampC);
 bool i32f_allowed();
 void col_range_exact(const HostInst &h, int64_t &lo, int64_t &hi);
 int64_t walked_energy_max(const HostInst &h);
 bool i16p_exact(HostInst &h);
 void i16p_fuse_el(HostInst &h);
+void center_rows(HostInst &h);
 bool i16p_group_ok(const HostInst &h);
 void i16p_step_form(HostInst &h, bool allow_grouped);
 bool i16p_allowed();

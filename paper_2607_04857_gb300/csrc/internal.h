@@ -142,6 +142,7 @@ struct Inst {
                           // packed column minima without a carry (the host proves the sums fit 16 bits)
     int32_t elmin;        // ACC_I16P with el_fused: a lower bound of every E_L value
     float geps;           // ACC_F32, grouped form: rounding allowance of a group's column updates
+    int32_t center[4];    // grouped integer scans: moved from E_L to the rows 0-3 (plan.cu: center_rows)
     int32_t limb;         // ACC_I64: > 0, energies on two limbs hi * 2^limb + lo (scan_i64.cu)
 };
 

@@ -426,6 +426,8 @@ __global__ void tables_kernel(const Inst *insts)
     auto m_entry = [&](long r, long j) {
         const int vr = B + (int)r;
         F acc = 0;
+        if constexpr (Tr<T>::kGrouped && !Tr<T>::kFloat)
+            acc = r < 4 ? (F)d.center[r] : (F)0;
         for (int b = 0; b < B; ++b)
             if ((j >> b) & 1)
                 acc += W[vr * n + b];
@@ -466,6 +468,8 @@ __global__ void tables_kernel(const Inst *insts)
                 if (!((g >> r) & 1))
                     continue;
                 acc += W[(B + r) * n + (B + r)];
+                if constexpr (Tr<T>::kGrouped && !Tr<T>::kFloat)
+                    acc -= r < 4 ? (F)d.center[r] : (F)0;
                 for (int r2 = r + 1; r2 < L; ++r2)
                     if ((g >> r2) & 1)
                         acc += W[(B + r) * n + (B + r2)];
