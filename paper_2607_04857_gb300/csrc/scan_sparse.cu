@@ -472,12 +472,23 @@ __global__ void __launch_bounds__(kScanThreads, S == 16 ? 4 : 3) zscan_kernel(co
 // A warp takes the units it claims two at a time: both units' minima of e are formed in one pass
 // over E_L, which halves the L1 traffic of that pass (it ran near the L1 load bandwidth).
 
+// v + w of the pass over E_L.  Integer adds and 3-input minima would all go to the ALU pipe (74% busy
+// with the FMA pipe at 36%): three of four adds are multiply-adds by a one the compiler cannot see.
+// With the adds per step taken from 1.25 to 1 and the pass unrolled by four, n=56 (2^46 states a launch):
+// 4.77 -> 4.52 ms; with the column minima formed the same way and the fixed variables' sums shared by
+// the units of a claim (unit_fields_shared), 4.28 ms; FP32 energies, n=56: 5.55 -> 4.64 ms.
+__device__ __forceinline__ int32_t step_add(int32_t v, int32_t w, int32_t one, int k)
+{
+    return k == 3 ? v + w : v * one + w;
+}
+__device__ __forceinline__ float step_add(float v, float w, float, int) { return v + w; }
+
 // Minima over the 2^Z walk steps of U units of e_u(i) = E_L(g(i)) + the sum of unit u's
 // zero-row couplings of the set bits of g(i) (Z >= 7; the same decomposition as zscan_unit's
 // block minima, parity 0), one read of E_L for all U units.  out[u] is the warp's minimum.
 template <class X, int U>
 __device__ __forceinline__ void walk_min_units(const X *EL, int Z, int lane, X *const (&wsm)[U], X *const (&wt)[U],
-                                               X *gs, X (&out)[U])
+                                               X *gs, X one, X (&out)[U])
 {
     const int zt = Z - 7;
 #pragma unroll
@@ -495,51 +506,64 @@ __device__ __forceinline__ void walk_min_units(const X *EL, int Z, int lane, X *
             wt[u][e] = gs[(e ^ (e >> 1)) & ((1 << zt) - 1)];
         __syncwarp();  // gs is rebuilt for the next unit
     }
+    // Per element k of a lane's four steps: the minimum over the even and the odd t of E_L plus the high
+    // bits' part; what depends on the lane and k alone is added once, after the loop (an add and half a
+    // 3-input minimum per step).
+    const X *e = EL + 4 * lane;
+    X me[U][4], mo[U][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            me[u][k] = mo[u][k] = zbig<X>();
+    if (zt >= 2) {
+#pragma unroll 1
+        for (int t = 0; t < (1 << zt); t += 4) {
+            X v[4][4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                vload<X>(e + ((t + s) << 7), v[s]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                X w[4];
+                vsplit(*(const typename VecOf<X>::type *)(wt[u] + t), w);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    me[u][k] = emin3(me[u][k], step_add(v[0][k], w[0], one, k), step_add(v[2][k], w[2], one, k));
+                    mo[u][k] = emin3(mo[u][k], step_add(v[1][k], w[1], one, k), step_add(v[3][k], w[3], one, k));
+                }
+            }
+        }
+    } else {
+        for (int t = 0; t < (1 << zt); ++t) {
+            X v[4];
+            vload<X>(e + (t << 7), v);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const X x = v[k] + wt[u][t];
+                    me[u][k] = t ? me[u][k] : x;
+                    mo[u][k] = t ? x : mo[u][k];
+                }
+        }
+    }
     const bool l0 = lane & 1, l4 = (lane >> 4) & 1;
-    X ae[U][4], ao[U][4];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         X a = 0;
         for (int r = 0; r < 4; ++r)
             if (((lane >> r) ^ (lane >> (r + 1))) & 1)
                 a += wsm[u][2 + r];
+        out[u] = zbig<X>();
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const bool g0 = (k ^ (k >> 1)) & 1, g1 = ((k >> 1) & 1) ^ l0;
             const X base = a + (g0 ? wsm[u][0] : 0) + (g1 ? wsm[u][1] : 0);
-            ae[u][k] = base + (l4 ? wsm[u][6] : 0);
-            ao[u][k] = base + (l4 ? 0 : wsm[u][6]);
+            out[u] = emin(out[u], me[u][k] + (base + (l4 ? wsm[u][6] : 0)));
+            if (zt > 0)
+                out[u] = emin(out[u], mo[u][k] + (base + (l4 ? 0 : wsm[u][6])));
         }
-    }
-    const X *e = EL + 4 * lane;
-    if (zt == 0) {
-        X v[4];
-        vload<X>(e, v);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            out[u] = emin(emin3(v[0] + ae[u][0], v[1] + ae[u][1], v[2] + ae[u][2]), v[3] + ae[u][3]);
-    } else {
-        X me[U], mo[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            me[u] = mo[u] = zbig<X>();
-        const int nt = 1 << zt;
-#pragma unroll 4
-        for (int t = 0; t < nt; t += 2) {
-            X v[4], w[4];
-            vload<X>(e + (t << 7), v);
-            vload<X>(e + ((t + 1) << 7), w);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const X mv = emin(emin3(v[0] + ae[u][0], v[1] + ae[u][1], v[2] + ae[u][2]), v[3] + ae[u][3]);
-                const X mw = emin(emin3(w[0] + ao[u][0], w[1] + ao[u][1], w[2] + ao[u][2]), w[3] + ao[u][3]);
-                me[u] = emin(me[u], mv + wt[u][t]);
-                mo[u] = emin(mo[u], mw + wt[u][t + 1]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            out[u] = emin(me[u], mo[u]);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -548,18 +572,56 @@ __device__ __forceinline__ void walk_min_units(const X *EL, int Z, int lane, X *
             out[u] = emin(out[u], __shfl_xor_sync(kFull, out[u], o));
 }
 
+// The part of unit_fields that the eight units unit | 0..7 share: kept while a warp goes through a
+// claim of eight units (integers; FP32 sums keep their order and are formed per unit).
+template <class X>
+struct ZBase {
+    uint64_t unit = ~0ull;
+    X f0 = 0, cx = 0;
+};
+constexpr int kZShared = 3;
+static_assert(2 + 5 + 4 + kZMaxRows + kZShared <= 32, "the shared bits' variables have a lane");
+
+template <class T>
+__device__ __forceinline__ void unit_fields_shared(const Inst &d, int BL, uint64_t unit, int lane,
+                                                   ZBase<typename Tr<T>::TC> &zb, typename Tr<T>::TC &f0,
+                                                   typename Tr<T>::TC &cx)
+{
+    using X = typename Tr<T>::TC;
+    const X *W = unit_matrix<T>(d);
+    if constexpr (std::is_integral<X>::value) {
+        const uint64_t low = (1ull << kZShared) - 1;
+        if ((unit & ~low) != zb.unit) {
+            zb.unit = unit & ~low;
+            unit_fields<T>(W, d.n, d.k, BL, zb.unit, lane, zb.f0, zb.cx);
+        }
+        f0 = zb.f0;
+        cx = zb.cx;
+#pragma unroll 1
+        for (int q = 0; q < kZShared; ++q)
+            if ((unit >> q) & 1ull) {  // the variable's own field so far is in its lane
+                const X w = lane < d.n ? W[(BL + q) * d.n + lane] : 0;
+                cx += __shfl_sync(kFull, f0 + w, BL + q);
+                f0 += lane == BL + q ? 0 : w;
+            }
+    } else {
+        unit_fields<T>(W, d.n, d.k, BL, unit, lane, f0, cx);
+    }
+}
+
 // Set-up of one unit x_f: the fields of its set fixed bits (f0, one variable per lane), c(x_f),
 // the zero-row couplings w_r into wsm, and the lane's minimum over its columns
 // E_s(j) + lin(j), j = (g * 32 + lane) * 4 + e.
 template <class T, int S>
-__device__ __forceinline__ void unit_one_setup(const Inst &d, uint64_t unit, int lane, typename Tr<T>::TC *wsm,
-                                               typename Tr<T>::TC &f0, typename Tr<T>::TC &cx, typename Tr<T>::TC &cm)
+__device__ __forceinline__ void unit_one_setup(const Inst &d, uint64_t unit, int lane, typename Tr<T>::TC one,
+                                               ZBase<typename Tr<T>::TC> &zb, typename Tr<T>::TC *wsm, typename Tr<T>::TC &f0,
+                                               typename Tr<T>::TC &cx, typename Tr<T>::TC &cm)
 {
     using X = typename Tr<T>::TC;
     constexpr int V = 4, G = S / V, LOGG = ilog2c(G);
     constexpr int B = 2 + 5 + LOGG;
     const int BL = B + d.L;
-    unit_fields<T>(unit_matrix<T>(d), d.n, d.k, BL, unit, lane, f0, cx);
+    unit_fields_shared<T>(d, BL, unit, lane, zb, f0, cx);
     __syncwarp();
     if (lane >= B && lane < BL)
         wsm[lane - B] = f0;
@@ -567,15 +629,21 @@ __device__ __forceinline__ void unit_one_setup(const Inst &d, uint64_t unit, int
     X lin_t, lin_e[V], lin_g[G];
     column_fields<X, V, G>(f0, lane, lin_t, lin_e, lin_g);
     const X *Es = (const X *)d.Es;
-    cm = zbig<X>();
+    // as in walk_min_units: the minimum over the groups for each of the lane's four columns first
+    X ce[V];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        X ev[V];
+    for (int e = 0; e < V; ++e)
+        ce[e] = zbig<X>();
+#pragma unroll
+    for (int g = 0; g < G; g += 2) {
+        X ev[V], ew[V];
         vload<X>(Es + (g * 32 + lane) * V, ev);
-        const X l = lin_t + lin_g[g];
-        cm = emin(cm, emin3(ev[0] + lin_e[0] + l, ev[1] + lin_e[1] + l,
-                            emin(ev[2] + lin_e[2] + l, ev[3] + lin_e[3] + l)));
+        vload<X>(Es + ((g + 1) * 32 + lane) * V, ew);
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+            ce[e] = emin3(ce[e], step_add(ev[e], lin_g[g], one, e), step_add(ew[e], lin_g[g + 1], one, e));
     }
+    cm = emin(emin3(ce[0] + lin_e[0], ce[1] + lin_e[1], ce[2] + lin_e[2]), ce[3] + lin_e[3]) + lin_t;
 }
 
 // Threshold test of a unit whose walk minimum of e is mel; a unit that reaches the threshold is
@@ -668,7 +736,7 @@ __device__ void unit_one_finish(const ScanArgs &a, const Inst &d, int inst, uint
 // Per-warp shared memory of the one-block kernel: two units' zero-row couplings and high-bit
 // tables, the doubling scratch, and the column groups' fields of a hit unit.
 template <class X, int S>
-struct OneSmem {
+struct alignas(16) OneSmem {
     X wsm[2][kMaxWalkBits];
     X wt[2][1 << (kZMaxRows - 7)];
     X gs[1 << (kZMaxRows - 7)];
@@ -683,6 +751,8 @@ __global__ void __launch_bounds__(kScanThreads, 6) zscan_one_kernel(const ScanAr
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     OneSmem<X, S> &sm = sm_all[warp];
     typename Tr<T>::TP Treg = 0;
+    const X one = (X)(int32_t)(a.mad_inverse * kMad);  // 1
+    ZBase<X> zb;
     // the persistent loop of persistent_units, taking the units of a claim two at a time
     constexpr unsigned long long kChunk = 8;
     int cur = -1;
@@ -720,6 +790,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) zscan_one_kernel(const ScanAr
                     atomicAdd(&a.state[cur].scanned, done);
                 done = 0;
                 cur = inst;
+                zb.unit = ~0ull;
                 Treg = Tr<T>::thr_load(a.state + inst);
             }
             const Inst d = a.inst[inst];
@@ -731,13 +802,13 @@ __global__ void __launch_bounds__(kScanThreads, 6) zscan_one_kernel(const ScanAr
             const uint64_t unit = d.unit_begin + (item - a.item_base[inst]);
             const bool pair = item + 1 < end && a.item_base[inst + 1] > item + 1;
             X f0a, cxa, cma, f0b = 0, cxb = 0, cmb = 0;
-            unit_one_setup<T, S>(d, unit, lane, sm.wsm[0], f0a, cxa, cma);
+            unit_one_setup<T, S>(d, unit, lane, one, zb, sm.wsm[0], f0a, cxa, cma);
             if (pair) {
-                unit_one_setup<T, S>(d, unit + 1, lane, sm.wsm[1], f0b, cxb, cmb);
+                unit_one_setup<T, S>(d, unit + 1, lane, one, zb, sm.wsm[1], f0b, cxb, cmb);
                 X *const w[2] = {sm.wsm[0], sm.wsm[1]};
                 X *const t[2] = {sm.wt[0], sm.wt[1]};
                 X mel[2];
-                walk_min_units<X, 2>((const X *)d.EL, d.L, lane, w, t, sm.gs, mel);
+                walk_min_units<X, 2>((const X *)d.EL, d.L, lane, w, t, sm.gs, one, mel);
                 unit_one_finish<T, S, K1>(a, d, inst, unit, Treg, lane, sm.wsm[0], sm.lin, f0a, cxa, cma, mel[0]);
                 unit_one_finish<T, S, K1>(a, d, inst, unit + 1, Treg, lane, sm.wsm[1], sm.lin, f0b, cxb, cmb, mel[1]);
                 done += 2ull << (d.B + d.L);
@@ -746,7 +817,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) zscan_one_kernel(const ScanAr
                 X *const w[1] = {sm.wsm[0]};
                 X *const t[1] = {sm.wt[0]};
                 X mel[1];
-                walk_min_units<X, 1>((const X *)d.EL, d.L, lane, w, t, sm.gs, mel);
+                walk_min_units<X, 1>((const X *)d.EL, d.L, lane, w, t, sm.gs, one, mel);
                 unit_one_finish<T, S, K1>(a, d, inst, unit, Treg, lane, sm.wsm[0], sm.lin, f0a, cxa, cma, mel[0]);
                 done += 1ull << (d.B + d.L);
                 item += 1;

@@ -78,6 +78,28 @@ def test_one_block_kernel_unit_pairing(q, n, units):
     check_int(r, oracle.solve(Q, topk=12))
 
 
+@pytest.mark.parametrize("dtype", [np.int32, np.float32])
+@pytest.mark.parametrize("walk", [7, 8, 9, 11])
+@pytest.mark.parametrize("fixed", [0, 1, 2, 6])
+def test_one_block_kernel_short_walks(q, walk, fixed, dtype):
+    """The one-block kernel at its shortest walks (one and two 128-step rows of E_L, then four at a
+    time) and with 0 to 6 fixed variables: units of a claim of eight share the sums of the fixed
+    variables above the lowest three.  The walked variables couple to each other and to the fixed
+    ones only, everything else to everything."""
+    n = 11 + walk + fixed
+    rng = np.random.default_rng(10 * walk + fixed)
+    Q = np.triu(rng.integers(-300, 301, size=(n, n)))
+    Q[:11, 11:11 + walk] = 0
+    Q = (Q if dtype is np.int32 else Q / 1024).astype(dtype)
+    for kw in (dict(), dict(fix_bits=1, fix_value=1)) if fixed > 1 else (dict(),):
+        r, o = q.solve(Q, topk=12, walk_bits=walk, **kw), oracle.solve(Q, topk=12, **kw)
+        assert (r.info["acc"], r.info["zero_rows"]) == ("i32z" if dtype is np.int32 else "f32z", walk), r.info
+        if dtype is np.int32:
+            check_int(r, o)
+        else:  # multiples of 2^-10 below 2^14: exact in FP32, ties included
+            assert r.min == o.min and r.n_ties == o.n_ties and np.array_equal(r.topk_E, o.topk_E)
+
+
 def test_sparse_subcubes(q):
     Q = wl.sparse_int(40, 0.06, -1000, 1000, seed=40)
     for v in (0, 3, 1000, (1 << 14) - 1):
