@@ -36,9 +36,10 @@ constexpr int kRegRows = 4;
 // pipe), 2- or 3-input mins, and the step form: 0, all adds first, then the min tree; 1, the adds
 // interleaved with the first level of the min tree (each triple of columns reduced as soon as its
 // adds are issued); 2, the grouped form (scan_grouped.cuh): groups of 16 steps skip the min tree
-// while a per-thread lower bound of the column minimum, moved by the steps' smallest column deltas,
-// proves that no column can reach the threshold.  The 8-byte
-// accumulators compile one variant: S = 16 with variant 0's register rows, blocks and min inputs.
+// while the columns' minimum over the group, formed once at its first state, proves that none
+// reaches the threshold; its integer columns take no add mode (group_updates).  FP64 compiles
+// variant 0 alone: S = 16 with its register rows, blocks and min inputs; int64 that and
+// kLimbVariant.
 constexpr int kScanVariants = 24;
 constexpr int kVariantCols[kScanVariants] = {32, 16, 16, 16, 16, 16, 32, 16, 16, 16, 16, 16,
                                              16, 16, 16, 16, 16, 16, 16, 16, 16, 16, 16, 16};

@@ -71,12 +71,12 @@ __device__ __forceinline__ void capped_add(uint32_t &x, uint32_t a)
 
 // The column updates of a skipped group.  FP32 adds are not reassociated.  Integer adds are: the
 // compiler would fold a run of them into one (or, as opaque instructions, in pairs into 3-input
-// adds), and the energies between would never be formed.  So a column's plain adds alternate with
-// multiply-adds by a run-time one, which no add next to them can be merged with, in a checkerboard
-// over steps and columns, so that every step feeds both integer pipes.  Measured per 16-column step
-// with the group's test: 18.1 cycles, all 240 updates issued (instruction count); 21.7 with
-// every second step's adds predicated instead, 24.3 with every add predicated, 29.3 for plain adds
-// with the min over the columns.
+// adds), and the energies between would never be formed.  So a column's capped adds alternate with
+// multiply-adds by kMad, which no add next to them can be merged with, in a checkerboard over steps
+// and columns, so that every step feeds both integer pipes.  All 240 updates of a group are issued
+// (instruction count).  A whole n=38 scan takes 19.7 cycles per 16-column step, tests and set-up
+// included; of the other forms measured, a skipped group alone took 21.7 with every second step's
+// adds predicated, 24.3 with every add predicated and 29.3 for plain adds with the min over the columns.
 template <class TC, int S, int ADDM, int PAR, int NR>
 __device__ __forceinline__ void group_updates(TC (&E)[S], const TC (&Mr)[NR][S])
 {
