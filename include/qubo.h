@@ -37,7 +37,9 @@ typedef enum { QUBO_I16 = 1, QUBO_I32 = 2, QUBO_F32 = 3, QUBO_F64 = 4 } qubo_dty
 /* Accumulator the scan ran in (reported in qubo_result.acc).  QUBO_ACC_F32: float Q scanned in
  * FP32, the running energies rebuilt from the tables every 2^10 walk steps (shorter when the
  * measured drift needs it; qubo_result.anchor_bits), every state within the candidate margin
- * rescored in FP64.  QUBO_ACC_I32F: integer energies held exactly in FP32 lanes, chosen when
+ * rescored in FP64; where the caller's margin has no room for the scan's rounding, a wider one of
+ * twice the worst-case rounding bound is taken (more candidates, the same answer).
+ * QUBO_ACC_I64: int64 energies, scanned on two 32-bit limbs when sum |U_ij| < 2^55.  QUBO_ACC_I32F: integer energies held exactly in FP32 lanes, chosen when
  * every value the run's plan holds in a lane stays below 2^24 in magnitude.  QUBO_ACC_I16P: integer energies held as two 16-bit lanes per 32-bit word,
  * chosen (before QUBO_ACC_I32F) when every column value of the run's plan provably lies in
  * [-32768, 32767].  QUBO_ACC_I32Z: int32 energies of a sparse instance, chosen first when the
@@ -156,7 +158,8 @@ typedef struct {
                                  the min over the columns while a lower bound of the column
                                  minimum proves the group holds no candidate (FP32, integers in
                                  FP32 lanes, int32: variants 20-23; packed 16-bit: 20 and 21;
-                                 every state's column add still runs); 0 otherwise */
+                                 int64 on two limbs: 1; every state's column add still runs); 0
+                                 otherwise */
 } qubo_result;
 
 /*

@@ -1044,7 +1044,7 @@ bool float_margin_ok(const HostInst &h, const Part &p, double margin)
 // the FP64 rescoring.  A wider margin only adds candidates.  When they are more than kProvenRecords
 // (dense low spectra, e.g. large penalty terms) the run ends early and the FP64 scan runs instead, as
 // without this attempt.  n=31, entries uniform in [-100, 100]: 0.19 ms of scan against 9.2 ms in FP64
-// (an FP64 add takes a warp 70 cycles on GB300), which three FP32 scans preceded.
+// (an FP64 add takes a warp about 75 cycles on GB300), which three FP32 scans preceded.
 constexpr unsigned long long kProvenRecords = 1ull << 16;
 int solve_proven(Workspace &ws, HostInst &h, const qubo_options &o, SolveCfg c, cudaStream_t stream, Part &p,
                  SolveStats &stats, double deadline, bool *done)

@@ -15,8 +15,8 @@
 // shared memory): the exact minimum over the group, with no slack but E_L's.  Groups that fail it
 // (n=36: 0.002% of them, n=48 Max-Cut 0.004%) are walked state by state.
 //
-// What bounds it (GB300, cycles per 16-column step per scheduler): eight f32x2 adds 16.1 (both halves
-// of the FMA pipe); sixteen int32 adds 16 when half of them issue to the FMA pipe's heavy half and
+// What bounds it (GB300, cycles per 16-column step per scheduler): eight f32x2 adds 17.4 (both halves
+// of the FMA pipe); sixteen int32 adds as long when half of them issue to the FMA pipe's heavy half and
 // half to the ALU pipe (group_updates).
 #pragma once
 
@@ -74,9 +74,9 @@ __device__ __forceinline__ void capped_add(uint32_t &x, uint32_t a)
 // adds), and the energies between would never be formed.  So a column's capped adds alternate with
 // multiply-adds by kMad, which no add next to them can be merged with, in a checkerboard over steps
 // and columns, so that every step feeds both integer pipes.  All 240 updates of a group are issued
-// (instruction count).  A whole n=38 scan takes 19.7 cycles per 16-column step, tests and set-up
-// included; of the other forms measured, a skipped group alone took 21.7 with every second step's
-// adds predicated, 24.3 with every add predicated and 29.3 for plain adds with the min over the columns.
+// (instruction count).  A whole n=38 scan takes 21.2 cycles per 16-column step, tests and set-up
+// included; of the other forms measured, a skipped group alone took 23.4 with every second step's
+// adds predicated, 26.2 with every add predicated and 31.6 for plain adds with the min over the columns.
 template <class TC, int S, int ADDM, int PAR, int NR>
 __device__ __forceinline__ void group_updates(TC (&E)[S], const TC (&Mr)[NR][S])
 {

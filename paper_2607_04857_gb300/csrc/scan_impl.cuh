@@ -511,7 +511,7 @@ __global__ void tables_kernel(const Inst *insts)
 // g_r = f_r + couplings of walked bit r to the lane bits, T(x) the couplings among the walked bits
 // (lane t holds T of pattern t).  Each state is one add to the running sum of g in Gray order and
 // one add of T, not O(n^2) adds: what bounds it is the set-up, and for float Q, summed in FP64 here,
-// the FP64 unit (an add takes a warp about 70 cycles).  A warp per item; with one warp per instance
+// the FP64 unit (an add takes a warp about 75 cycles).  A warp per item; with one warp per instance
 // that summed every state on its own, 4096 states (n = 12) took 306 us.
 template <class T>
 __device__ void small_unit(const ScanArgs &a, const Inst &d, int inst, uint64_t chunk, int lane)
