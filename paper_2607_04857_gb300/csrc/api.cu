@@ -1216,12 +1216,16 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
     return QUBO_OK;
 }
 
-// A batched instance solved again alone because its FP32 margin does not hold.
-int solve_alone(Workspace &ws, HostInst &h, int topk, size_t cap, cudaStream_t stream, Part &p, SolveStats &stats)
+// A batched instance solved again alone: its records overflowed the shared buffer, or its FP32 margin
+// does not hold.  A float instance takes the whole chain of solve_one either way: an overflowed run says
+// nothing about the margin of the next one.
+int solve_alone(Workspace &ws, HostInst &h, const SolveCfg &c, cudaStream_t stream, Part &p, SolveStats &stats)
 {
+    if (!h.is_float)
+        return solve_range(ws, h, 0, 0, c, stream, p, stats, 0.0);
     qubo_options o{};
-    o.topk = topk;
-    return solve_one(ws, h, o, cap, stream, p, stats);
+    o.topk = c.K;
+    return solve_one(ws, h, o, c.cap, stream, p, stats);
 }
 
 void fill_plan_info(const HostInst &h, const SolveStats &stats, double t0, qubo_result *info)
@@ -1500,10 +1504,8 @@ int batch_parts(Workspace &ws, std::vector<HostInst> &hs, const std::vector<int>
         if (p.overflow || !float_margin_ok(h, p, c.margin)) {
             // rare: this instance overflowed the shared candidate buffer, or its FP32 margin does not
             // hold; solve it alone
-            const bool overflow = p.overflow;
             p = Part();
-            if ((st = overflow ? solve_range(ws, h, 0, 0, c, stream, p, stats, 0.0)
-                               : solve_alone(ws, h, topk, cap, stream, p, stats)))
+            if ((st = solve_alone(ws, h, c, stream, p, stats)))
                 return st;
         }
         if (p.scanned != (1ull << h.n) || !p.has)
@@ -2354,10 +2356,8 @@ int qubo_batch_fetch(qubo_batch *b, void *out_min, uint64_t *out_states, uint64_
             if ((st = sw->init(dev)))
                 return st;
             HostInst hc = h;
-            const bool overflow = p.overflow;
             p = Part();
-            if ((st = overflow ? solve_range(*sw, hc, 0, 0, c, j.stream, p, st2, 0.0)
-                               : solve_alone(*sw, hc, b->topk, b->cap, j.stream, p, st2)))
+            if ((st = solve_alone(*sw, hc, c, j.stream, p, st2)))
                 return st;
         }
         if (p.scanned != (1ull << h.n) || !p.has)

@@ -1,0 +1,58 @@
+"""Float instances of a batch whose records overflow the shared buffer or whose magnitudes leave the
+candidate margin no room: solved again alone, with the results of the CPU oracle (FP64)."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def q():
+    import paper_2607_04857_gb300 as q
+
+    q.load_library()
+    return q
+
+
+def twins(n, pairs, scale, seed):
+    """A float matrix of whole numbers in which variables v and v + n/2 (v < pairs) couple alike to all
+    others and exclude each other: exact ties in FP64 whose FP32 energies differ by their rounding."""
+    rng = np.random.default_rng(seed)
+    A = np.triu(rng.integers(-scale, scale + 1, size=(n, n)), 1)
+    A = A + A.T
+    d = rng.integers(-scale, scale + 1, size=n)
+    of = np.arange(n)
+    of[n // 2:n // 2 + pairs] -= n // 2  # a twin has its original's row
+    A, d = A[np.ix_(of, of)], d[of]
+    for v in range(pairs):
+        t = v + n // 2
+        A[v, t] = A[t, v] = 4 * scale
+        d[v] = d[t] = d[v] - 3 * scale
+    return (np.triu(A, 1) + np.diag(d)).astype(np.float64)
+
+
+def check(r, o):
+    assert r.min == o.min and r.n_ties == o.n_ties
+    assert np.array_equal(r.ties, o.ties) and np.array_equal(r.topk, o.topk) and np.array_equal(r.topk_E, o.topk_E)
+
+
+@pytest.mark.parametrize("scale", [10, 10**4, 10**7])
+@pytest.mark.parametrize("graph", [False, True])
+def test_overflow_beside_large_magnitudes(q, scale, graph, monkeypatch):
+    """One instance of nothing but ties fills the buffer; the others lose records and are solved again,
+    with FP32's rounding at scale 10^7 a thousand times the default margin."""
+    Qs = [np.zeros((16, 16))] + [twins(22, 5, scale, seed) for seed in range(6)]
+    monkeypatch.setenv("QUBO_MAX_RECORDS", "2000")
+    if graph:
+        b = q.Batch(Qs, topk=20, states_cap=64)
+        b.run()
+        rs = b.fetch()
+    else:
+        rs = q.solve_batched(Qs, topk=20, states_cap=64)
+    assert max(r.info["passes"] for r in rs) > 1
+    for Q, r in zip(Qs, rs):
+        check(r, oracle.solve(Q, topk=20, cap=64))
+    if graph:
+        b.close()
