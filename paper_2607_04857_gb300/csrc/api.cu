@@ -130,6 +130,7 @@ struct Part {
     std::vector<std::pair<int64_t, uint64_t>> topi; // int
     uint64_t scanned = 0, candidates = 0;
     double drift = 0.0, err = 0.0;
+    double slack = 0.0;  // float_slack of the FP32 scans among the runs merged into this part, 0 without
     bool overflow = false;
     uint64_t dbg = 0;  // QUBO_DEBUG builds: site of the first failed device check
     // energy-window mode: every state with E <= min + window, (E, code) ascending (energies as
@@ -156,6 +157,7 @@ Part merge_parts(const Part &a, const Part &b, size_t cap, int K)
     o.candidates = a.candidates + b.candidates;
     o.drift = std::max(a.drift, b.drift);
     o.err = std::max(a.err, b.err);
+    o.slack = std::max(a.slack, b.slack);
     o.overflow = a.overflow || b.overflow;
     if (part_eq_min(a, b)) {
         o.min_i = a.min_i;
@@ -815,6 +817,19 @@ int job_enqueue_finalize(Workspace &ws, Job &j, unsigned long long max_count, un
     return QUBO_OK;
 }
 
+// FP32 scans: the candidate margin must cover twice the measured drift plus the rounding of the
+// per-step threshold arithmetic (a few FP32 operations on values bounded by beta; the factored
+// scan's E_L plus up to 14 zero-row couplings, more).  Otherwise the caller rescans with a
+// shorter walk, the dense FP32 scan, a proven margin, or FP64.  Direct evaluation sums in FP64.
+double float_slack(Acc acc, double beta)
+{
+    return (acc == ACC_F32Z ? 32.0 : 8.0) * std::ldexp(1.0, -24) * (1.0 + beta);
+}
+bool float_margin_ok(const Part &p, double margin)
+{
+    return p.slack == 0.0 || 2.0 * p.drift + p.slack < margin;
+}
+
 Part part_from(const Down &d, const Job &j, int i);
 
 // After the stream has finished: timings and per-instance results from the staging buffer.
@@ -859,6 +874,8 @@ Part part_from(const Down &d, const Job &j, int i)
         p.candidates = d.sts[i].nrec;
         p.drift = ubits_to_double(d.sts[i].drift);
         p.err = ubits_to_double(d.sts[i].err);
+        const HostInst &h = *j.insts[i];
+        p.slack = (j.acc == ACC_F32 || j.acc == ACC_F32Z) && !h.small ? float_slack(j.acc, h.beta) : 0.0;
         p.overflow = d.sts[i].dropped > 0;
         p.dbg = d.sts[i].dbg;
     }
@@ -1023,21 +1040,6 @@ int solve_range(Workspace &ws, HostInst &h, int fix_bits, uint64_t fix_value, co
     return QUBO_OK;
 }
 
-// FP32 scans: the candidate margin must cover twice the measured drift plus the rounding of the
-// per-step threshold arithmetic (a few FP32 operations on values bounded by beta; the factored
-// scan's E_L plus up to 14 zero-row couplings, more).  Otherwise the caller rescans with a
-// shorter walk, the dense FP32 scan, a proven margin, or FP64.  Direct evaluation sums in FP64.
-double float_slack(const HostInst &h)
-{
-    return (h.acc == ACC_F32Z ? 32.0 : 8.0) * std::ldexp(1.0, -24) * (1.0 + h.beta);
-}
-bool float_margin_ok(const HostInst &h, const Part &p, double margin)
-{
-    if ((h.acc != ACC_F32 && h.acc != ACC_F32Z) || h.small)
-        return true;
-    return 2.0 * p.drift + float_slack(h) < margin;
-}
-
 // A float instance whose magnitudes leave the caller's candidate margin no room for an FP32 scan's
 // rounding (entries of order 100 at n = 30) is scanned in FP32 all the same, with a wider margin: twice
 // the worst-case rounding bound of the run's plan, which proves that every state of the answer reaches
@@ -1067,7 +1069,7 @@ int solve_proven(Workspace &ws, HostInst &h, const qubo_options &o, SolveCfg c, 
     p = Part();
     if ((st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))
         return st;
-    *done = !p.overflow && h.acc == ACC_F32 && float_margin_ok(h, p, m);
+    *done = !p.overflow && h.acc == ACC_F32 && float_margin_ok(p, m);
     return QUBO_OK;
 }
 
@@ -1172,18 +1174,18 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
     int st;
     const bool fp32 = h.acc == ACC_F32 && !(c.flags & (QUBO_FLAG_PLAIN | QUBO_FLAG_RIGOROUS));
     bool done = false, tried = false;
-    if (fp32 && !(2.0 * float_slack(h) < c.margin)) {  // little or no room for a drift in the margin
+    if (fp32 && !(2.0 * float_slack(h.acc, h.beta) < c.margin)) {  // little or no room for a drift in the margin
         tried = true;
         if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
             return st;
         if (!done && !h.small)
-            h.acc = float_slack(h) < c.margin ? ACC_F32 : ACC_F64;
+            h.acc = float_slack(h.acc, h.beta) < c.margin ? ACC_F32 : ACC_F64;
     }
     if (!done && (st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))
         return st;
     // FP32 drift above the margin's budget: take a proven margin with a shorter re-anchoring period; when
     // that gives up, shorten the period further, and as a last resort rescan in FP64.
-    while (!done && !float_margin_ok(h, p, c.margin)) {
+    while (!done && !float_margin_ok(p, c.margin)) {
         const int period = std::min(h.anchor_bits, h.L);
         if (h.acc == ACC_F32Z) {  // the dense FP32 scan next
             h.no_factored = true;
@@ -1501,7 +1503,7 @@ int batch_parts(Workspace &ws, std::vector<HostInst> &hs, const std::vector<int>
         const int i = order[r];
         Part &p = run_parts[r];
         HostInst &h = hs[i];
-        if (p.overflow || !float_margin_ok(h, p, c.margin)) {
+        if (p.overflow || !float_margin_ok(p, c.margin)) {
             // rare: this instance overflowed the shared candidate buffer, or its FP32 margin does not
             // hold; solve it alone
             p = Part();
@@ -2139,7 +2141,7 @@ int qubo_problem_fetch(qubo_problem *p, void *out_min, uint64_t *out_states, siz
         return st;
     Part part = parts[0];
     const size_t cap = std::min<size_t>(states_cap, p->job.cap);
-    if (part.overflow || !float_margin_ok(p->h, part, p->job.margin) || states_cap > p->job.cap) {
+    if (part.overflow || !float_margin_ok(part, p->job.margin) || states_cap > p->job.cap) {
         // repeat through the splitting path (exact, uses this problem's workspace)
         qubo_options o = p->opt;
         o.fix_bits = p->fix_bits;
@@ -2302,7 +2304,7 @@ int qubo_batch_fetch(qubo_batch *b, void *out_min, uint64_t *out_states, uint64_
         const InstState &sts = d.sts[r];
         const double drift = ubits_to_double(sts.drift);
         const bool fast = res.has && sts.dropped == 0 && sts.scanned == (1ull << h.n) &&
-                          (h.acc != ACC_F32 || 2.0 * drift + 8.0 * std::ldexp(1.0, -24) * (1.0 + h.beta) < c.margin);
+                          (h.acc != ACC_F32 || 2.0 * drift + float_slack(h.acc, h.beta) < c.margin);
         qubo_result *inf = info ? info + i : nullptr;
         if (fast) {
             // common case: copy straight from the staging buffer
@@ -2345,7 +2347,7 @@ int qubo_batch_fetch(qubo_batch *b, void *out_min, uint64_t *out_states, uint64_
         }
         Part p = part_from(d, j, r);
         SolveStats st2 = stats;
-        if (p.overflow || !float_margin_ok(h, p, c.margin)) {
+        if (p.overflow || !float_margin_ok(p, c.margin)) {
             // rare: solve this instance alone on the shared workspace (the graph's is fixed)
             Workspace *sw = nullptr;
             if ((st = resolve_device(&sw)))

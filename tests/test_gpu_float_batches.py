@@ -56,3 +56,23 @@ def test_overflow_beside_large_magnitudes(q, scale, graph, monkeypatch):
         check(r, oracle.solve(Q, topk=20, cap=64))
     if graph:
         b.close()
+
+
+def test_every_part_of_a_split_range_keeps_to_the_margin(q, monkeypatch):
+    """Eight low variables whose fields the six top ones cancel when all are set: the sub-cube of the
+    top ones set holds the minimum 2^8 times, overflows and is split down to direct evaluation (FP64),
+    while the other parts are scanned in FP32 (factored), whose rounding at 10^6 is beyond the margin."""
+    scale, rng = 10**6, np.random.default_rng(0)
+    Q = np.zeros((20, 20))
+    Q[np.arange(8), np.arange(8)] = 6 * scale
+    Q[:8, 14:] = -scale
+    Q[8:, 8:] = np.triu(rng.integers(-scale, scale + 1, size=(12, 12)))
+    Q[np.arange(14, 20), np.arange(14, 20)] -= 4 * scale
+    assert oracle.solve(Q).n_ties == 256 and q.plan_query(Q)["acc"] == "f32z"
+    monkeypatch.setenv("QUBO_MAX_RECORDS", "64")
+    p = q.Problem(Q, topk=8)
+    p.run()
+    r = p.fetch()
+    p.close()
+    check(r, oracle.solve(Q, topk=8))
+    assert r.info["acc"] == "f64", r.info
