@@ -820,10 +820,17 @@ int job_enqueue_finalize(Workspace &ws, Job &j, unsigned long long max_count, un
 // FP32 scans: the candidate margin must cover twice the measured drift plus the rounding of the
 // per-step threshold arithmetic (a few FP32 operations on values bounded by beta; the factored
 // scan's E_L plus up to 14 zero-row couplings, more).  Otherwise the caller rescans with a
-// shorter walk, the dense FP32 scan, a proven margin, or FP64.  Direct evaluation sums in FP64.
+// shorter walk, the dense FP32 scan, a proven margin, or FP64.  Direct evaluation sums in FP64, but
+// its records hold FP32 energies: beyond FP32's range, infinities.
+constexpr double kFp32Beta = 1e30;  // energies an FP32 scan is given
 double float_slack(Acc acc, double beta)
 {
     return (acc == ACC_F32Z ? 32.0 : 8.0) * std::ldexp(1.0, -24) * (1.0 + beta);
+}
+double scan_slack(Acc acc, const HostInst &h)
+{
+    const bool fp32 = acc == ACC_F32 || acc == ACC_F32Z;
+    return fp32 && !(h.small && h.beta < kFp32Beta) ? float_slack(acc, h.beta) : 0.0;
 }
 bool float_margin_ok(const Part &p, double margin)
 {
@@ -874,8 +881,7 @@ Part part_from(const Down &d, const Job &j, int i)
         p.candidates = d.sts[i].nrec;
         p.drift = ubits_to_double(d.sts[i].drift);
         p.err = ubits_to_double(d.sts[i].err);
-        const HostInst &h = *j.insts[i];
-        p.slack = (j.acc == ACC_F32 || j.acc == ACC_F32Z) && !h.small ? float_slack(j.acc, h.beta) : 0.0;
+        p.slack = scan_slack(j.acc, *j.insts[i]);
         p.overflow = d.sts[i].dropped > 0;
         p.dbg = d.sts[i].dbg;
     }
@@ -1052,7 +1058,7 @@ int solve_proven(Workspace &ws, HostInst &h, const qubo_options &o, SolveCfg c, 
                  SolveStats &stats, double deadline, bool *done)
 {
     *done = false;
-    if (!(h.beta < 1e30))  // FP32 range
+    if (!(h.beta < kFp32Beta))
         return QUBO_OK;
     h.acc = ACC_F32;
     h.no_factored = true;
@@ -1178,7 +1184,7 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
         tried = true;
         if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
             return st;
-        if (!done && !h.small)
+        if (!done && scan_slack(h.acc, h) > 0.0)
             h.acc = float_slack(h.acc, h.beta) < c.margin ? ACC_F32 : ACC_F64;
     }
     if (!done && (st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))

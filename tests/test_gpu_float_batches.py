@@ -76,3 +76,20 @@ def test_every_part_of_a_split_range_keeps_to_the_margin(q, monkeypatch):
     p.close()
     check(r, oracle.solve(Q, topk=8))
     assert r.info["acc"] == "f64", r.info
+
+
+@pytest.mark.parametrize("n", [1, 6, 11, 12, 16])
+def test_entries_beyond_fp32(q, n):
+    """Entries of 10^39 on every path, directly evaluated sizes among them: FP64 decides, and no
+    infinite energy enters the records or the reported rounding error."""
+    Q = np.random.default_rng(n).uniform(-1e39, 1e39, (n, n))
+    o = oracle.solve(Q, topk=2, cap=64)
+    b, p = q.Batch([Q, Q], topk=2), q.Problem(Q, topk=2)
+    b.run()
+    p.run()
+    rs = [q.solve(Q, topk=2), q.solve(Q, topk=2, rigorous=True), *q.solve_batched([Q, Q], topk=2), *b.fetch(), p.fetch()]
+    for r in rs:
+        check(r, o)
+        assert r.info["fp32_max_abs_err"] <= 1e-9 * abs(o.min), r.info
+    b.close()
+    p.close()
