@@ -1289,8 +1289,8 @@ int batch_walk(Acc acc, int variant, const HostInst &h, int wmax, const int (&tu
     const int rmin = variant_reg_rows(h) + 1;
     if (h.n - B < rmin)
         return 0;
-    const int tw = tuned[h.n];
-    if (tw >= rmin && tw <= std::min(kMaxWalkBits, h.n - B))
+    const int tw = tuned[h.n], tmax = acc == ACC_I64 && variant == kLimbVariant ? kLimbMaxWalkBits : kMaxWalkBits;
+    if (tw >= rmin && tw <= std::min(tmax, h.n - B))
         return tw;
     return std::max(rmin, std::min(wmax, h.n - B));
 }

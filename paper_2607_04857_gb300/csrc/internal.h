@@ -72,9 +72,10 @@ constexpr int kPackedMinBlocks[kScanVariants] = {3, 3, 3, 4, 4, 2, 2, 4, 3, 4, 3
 constexpr int kPackedAddMode[kScanVariants] = {0, 3, 2, 0, 3, 0, 3, 3, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 3, 2, 0, 0, 0, 0};
 constexpr int kPackedInterleave[kScanVariants] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 0, 1, 1, 1, 1, 2, 2, 3, 3};
 // The 8-byte accumulators have variant 0; int64 also the grouped scan on two 32-bit limbs
-// (scan_i64.cu) for energies below 2^55, which keeps four register rows.
+// (scan_i64.cu) for energies below 2^55, which keeps four register rows.  Its group test allows for the
+// low limbs of a column's base and of as many set rows as a walk has, at most kLimbMaxWalkBits.
 constexpr int kLimbVariant = 1;
-constexpr int kLimbMaxShift = 26;
+constexpr int kLimbMaxWalkBits = 14;
 // Whether a plan's scan kernel runs the grouped form.
 constexpr bool grouped_form(Acc acc, int variant)
 {

@@ -156,6 +156,7 @@ int variant_reg_rows(const HostInst &h)
 // Longest walk of an accumulator's plans.
 static int max_walk(Acc acc, bool grouped)
 {
+    static_assert(kGroupedMaxWalkBits <= kLimbMaxWalkBits, "the two-limb scan's own walks");
     return acc == ACC_F32       ? kFloatMaxWalkBits
            : acc == ACC_I32F    ? kI32FMaxWalkBits
            : acc_factored(acc) ? kZMaxWalkBits
@@ -218,7 +219,8 @@ int plan(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bi
     else
         L = std::max(rc + 1, std::min(max_walk(h.acc, false), free_bits - h.B - kTargetUnitsLog2));
     const int k = n - h.B - L;
-    if (L < rc + 1 || L > kMaxWalkBits || k < fix_bits || k > 63)
+    const int lmax = h.acc == ACC_I64 && h.variant == kLimbVariant ? kLimbMaxWalkBits : kMaxWalkBits;
+    if (L < rc + 1 || L > lmax || k < fix_bits || k > 63)
         return QUBO_ERR_ARG;
     h.L = L;
     h.k = k;
@@ -742,7 +744,7 @@ static int plan_uncentered(HostInst &h, int fix_bits, uint64_t fix_value, int sp
         // the two-limb kernel where its walk (at least five bits) fits
         const int bits = h.n - fix_bits - acc_suffix_bits(h.acc, 0);
         const int L = split_k > 0 ? h.n - acc_suffix_bits(h.acc, 0) - split_k : walk_bits > 0 ? walk_bits : bits;
-        h.variant = h.acc == ACC_I64 && L >= 5 && L <= (split_k > 0 || walk_bits > 0 ? kGroupedMaxWalkBits : L) &&
+        h.variant = h.acc == ACC_I64 && L >= 5 && L <= (split_k > 0 || walk_bits > 0 ? kLimbMaxWalkBits : L) &&
                             limb_shift(h) > 0 ? kLimbVariant : 0;
     }
     if (h.acc == ACC_I16P)

@@ -9,13 +9,15 @@ namespace {
 // A column's energy is held as hi * 2^s + lo, two int32 values that are updated separately: a table
 // row is split once into hi and lo (|lo| <= 2^(s-1)), and the walk adds the halves without carrying
 // from one to the other.  The lo of a column is then the sum of the lo of its base and of at most
-// 14 set rows, |lo| <= 15 * 2^(s-1) < 8 * 2^s, and with s = max(1, ceil(log2 beta) - 29) <= 26 both
-// limbs stay below 2^30 (beta < 2^55).  A state costs two int32 updates, no 64-bit minimum: the group
+// kLimbMaxWalkBits = 14 set rows, |lo| <= 15 * 2^(s-1) < 8 * 2^s, and with s = max(1, ceil(log2 beta) - 29)
+// <= 26 both limbs stay below 2^30 (beta < 2^55).  A state costs two int32 updates, no 64-bit minimum: the group
 // test of scan_grouped.cuh runs on the hi limbs alone, E > u - min E_L being certain when
-// hi > ((u - min E_L) >> s) + 8.  Groups it cannot clear are walked state by state in int64.
+// hi > ((u - min E_L) >> s) + 8 (at 16 set rows a group that holds the minimum can pass it).  Groups it cannot clear are walked state by state in int64.
 // What bounds it: the two integer pipes, 32 updates per 16-column step (two limbs).  n=34, entries up to
 // 2^30: the plain kernel (64-bit adds and minima, 217 cycles per step) takes 5.8 ms, this one 1.35 ms (51).
 constexpr int kLimbCols = 16, kLimbRows = 4;
+constexpr int kLimbSlack = 8;  // of a hi limb against the energy, in units of 2^s
+static_assert(kLimbMaxWalkBits + 1 < 2 * kLimbSlack, "the sum of the low limbs");
 
 __device__ __forceinline__ void split_limbs(int64_t v, int s, int32_t &hi, int32_t &lo)
 {
@@ -125,7 +127,7 @@ __device__ __forceinline__ void scan_unit_limbs(const ScanArgs &a, const Inst &d
             }
             const int i = i0 + t;
             const int64_t el = ELp[i], tp = u - el;
-            if (!__any_sync(kFull, (int64_t)tree_min<int32_t, 3, S>(Eh) <= (tp >> s) + 8))
+            if (!__any_sync(kFull, (int64_t)tree_min<int32_t, 3, S>(Eh) <= (tp >> s) + kLimbSlack))
                 continue;
             unsigned mask = 0;
 #pragma unroll
@@ -150,7 +152,7 @@ __device__ __forceinline__ void scan_unit_limbs(const ScanArgs &a, const Inst &d
     };
 
     const int ngrp = 1 << (L - 4);
-    if (!QUBO_DCHECK(L >= RC + 1 && L <= kMaxWalkBits, st, 9))
+    if (!QUBO_DCHECK(L >= RC + 1 && L <= kLimbMaxWalkBits, st, 9))
         return;
 #pragma unroll 1
     for (int g = 0; g < ngrp; ++g) {
@@ -174,7 +176,7 @@ __device__ __forceinline__ void scan_unit_limbs(const ScanArgs &a, const Inst &d
             P += sg * sm.wsm[row];
             u = Treg + mu - P;
         }
-        const int64_t limit = ((u - elg) >> s) + 8;
+        const int64_t limit = ((u - elg) >> s) + kLimbSlack;
         if (!__all_sync(kFull, (int64_t)tree_min<int32_t, 3, S>(Eh) + (odd ? Dgrp[1] : Dgrp[0]) > limit)) {
             int32_t low[S];
             static_for<G>([&](auto cc) {

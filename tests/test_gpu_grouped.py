@@ -240,3 +240,29 @@ def test_two_limbs_ties_window_batch(q):
     for M, r in zip(insts, q.solve_batched(insts, topk=4)):
         assert r.info["acc"] == "i64"
         check(r, oracle.solve(M, topk=4, cap=64))
+
+
+@pytest.mark.parametrize("walk", [13, 14, 15, 16])
+def test_two_limbs_longest_walk(q, walk, tmp_path):
+    """A minimum whose base and walked rows all have the lowest low limb: the sum of `walk` of them and
+    the base's.  A batch takes an installed plan's walk up to the 14 rows the group test allows for."""
+    n = 9 + walk + 2
+    Q = np.zeros((n, n), dtype=np.int32)
+    Q[0, 0] = Q[0, 9:9 + walk] = -(1 << 30) + 32
+    Q[1, 1], Q[9 + walk, 9 + walk], Q[10 + walk, 10 + walk] = 5, 77, 1000
+    path = str(tmp_path / "plans")
+    q.autotune_batched([wl.upper_int(16, -90, 90, seed=k, dtype=np.int16) for k in range(2)])
+    q.autotune_save(path)
+    device = open(path).read().split("\n")[1].split("\t")[:2]
+    q.autotune_clear()
+    with open(path, "w") as f:
+        f.write("qubo-autotune 1\n" + "\t".join(device + ["2", str(-n), "1", str(walk)]) + "\n")
+    assert q.autotune_load(path) == 1
+    try:
+        rs = q.solve_batched([Q, Q], topk=3)
+    finally:
+        q.autotune_clear()
+    for r in rs:
+        assert r.info["acc"] == "i64" and r.info["grouped"] == 1, r.info
+        assert r.info["walk_bits"] == walk if walk <= 14 else r.info["walk_bits"] <= 14, r.info
+        check(r, oracle.solve(Q, topk=3, cap=64))
