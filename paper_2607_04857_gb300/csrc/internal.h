@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "zscan.h"
@@ -100,6 +102,16 @@ constexpr bool packed_fused_only(int variant) { return variant >= 0 && variant <
 // Odd multiplier of the grouped form's integer multiply-adds (scan_grouped.cuh) and its inverse.
 constexpr uint32_t kMad = 0x9e3779b1u, kMadInverse = 0x0e8b2f51u;
 static_assert(kMad * kMadInverse == 1u, "the inverse of kMad modulo 2^32");
+// x + sign * factor * kept, modulo 2^32 for integers: factor * kept is the plain row value, but as a
+// product of two 32-bit words, whose signed form would overflow.
+template <class TC>
+__host__ __device__ constexpr TC add_kept_row(TC x, TC sign, TC factor, TC kept)
+{
+    if constexpr (std::is_integral_v<TC>)
+        return (TC)((uint32_t)x + (uint32_t)sign * (uint32_t)factor * (uint32_t)kept);
+    else
+        return x + sign * factor * kept;
+}
 // Threads per block of the scan kernel (4 warps; every warp owns one work unit at a time).
 constexpr int kScanThreads = 128;
 // Longest Gray walk inside one work unit (also the FP32 re-anchoring period).

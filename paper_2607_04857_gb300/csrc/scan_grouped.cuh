@@ -327,7 +327,7 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
                     const int q = g * V + e;
-                    low[q] = add_down(odd ? E[q] - mad_factor<TC>(3, q) * Mr[3][q] : E[q], nv[e]);
+                    low[q] = add_down(odd ? add_kept_row(E[q], (TC)-1, mad_factor<TC>(3, q), Mr[3][q]) : E[q], nv[e]);
                 }
             }
             return (DB)tree_min<TC, 3, S>(low);
@@ -382,7 +382,7 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
                 constexpr int e = decltype(ec)::value, q = g * V + e;
                 static_for<(NR < RC ? NR : RC)>([&](auto rc) {
                     constexpr int r = decltype(rc)::value;
-                    x[q] = x[q] + sr[r] * mad_factor<TC>(r, q) * Mr[r][q];
+                    x[q] = add_kept_row(x[q], sr[r], mad_factor<TC>(r, q), Mr[r][q]);
                 });
                 if constexpr (NG > 1)
                     x[q] = x[q] + sr[RC] * mv[e];
@@ -450,7 +450,7 @@ __device__ __forceinline__ void scan_unit_grouped(const ScanArgs &a, const Inst 
                         if (row == r)
                             static_for<S>([&](auto qc) {
                                 constexpr int q = decltype(qc)::value;
-                                E[q] = E[q] + sg * mad_factor<TC>(r, q) * Mr[r][q];
+                                E[q] = add_kept_row(E[q], sg, mad_factor<TC>(r, q), Mr[r][q]);
                             });
                     });
                 }

@@ -4,10 +4,15 @@ thread's exact column minimum m is taken, and over the group's next 15 steps (re
 the minimum must never fall below m + D, where D is the smallest running sum of each step's
 smallest column move.  E_L's group minimum completes the test.  A wrong sign pattern, a dropped
 coupling to the fixed bits or a running sum taken over the wrong steps fails these checks."""
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
 from paper_2607_04857_gb300 import workloads as wl
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def columns_over_walk(U, B, L, fixed):
@@ -125,3 +130,35 @@ def test_smallest_offset_bounds_every_column(seed):
         least = min((start + sum(((p >> r) & 1) * rows[r] for r in range(4))).min() for p in range(16))
         assert first.min() + D <= least
         assert D >= group_bound(rows, np.zeros(4, dtype=np.int64), par)
+
+
+def test_kept_rows_add_without_signed_overflow(tmp_path):
+    """A register row kept divided by kMad comes back as the plain row, in arithmetic that is defined for
+    every 32-bit word: signed overflow traps here."""
+    src = tmp_path / "rows.cpp"
+    src.write_text("""
+#include "internal.h"
+using namespace qubo;
+int main()
+{
+    uint32_t s = 12345;
+    for (int i = 0; i < 100000; ++i) {
+        s = s * 1664525u + 1013904223u;
+        const int32_t row = (int32_t)s >> (2 + i % 28), x = (int32_t)(s * 2654435761u) >> (2 + i % 5);
+        const int32_t kept = (int32_t)((uint32_t)row * kMadInverse);
+        for (int32_t sign = -1; sign <= 1; ++sign)
+            if (add_kept_row<int32_t>(x, sign, (int32_t)kMad, kept) != x + sign * row ||
+                add_kept_row<int32_t>(x, sign, 1, row) != x + sign * row)
+                return 1;
+        if (add_kept_row<float>(0.5f, -1.0f, 1.0f, 3.0f) != -2.5f)
+            return 2;
+    }
+    return 0;
+}
+""")
+    csrc = os.path.join(ROOT, "paper_2607_04857_gb300", "csrc")
+    exe = str(tmp_path / "rows")
+    subprocess.run(["g++", "-std=c++20", "-O1", "-fsanitize=signed-integer-overflow", "-fsanitize-undefined-trap-on-error",
+                    "-I", csrc, "-I", os.path.join(ROOT, "include"), "-I", "/usr/local/cuda/include", str(src), "-o", exe],
+                   check=True)
+    assert subprocess.run([exe]).returncode == 0
