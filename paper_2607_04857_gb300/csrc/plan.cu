@@ -899,7 +899,7 @@ namespace host {
 //   Ecol  = Ecol0 + ((1 + u)^t - 1) (Cc + Ecol0)                    t = 2^a steps since the anchor
 //   EP0   = (u + (k + 8) u64) bF + sum_{r >= RC} (u + k u64) rF(r)  c(x_f) and the couplings w_r,
 //         + (L - RC) u CP                                         each rounded once; re-anchoring
-//   EP    = EP0 + ((1 + u)^(t / 2^(RC+1) + 1) - 1) (CP + EP0)        one add per row-RC-or-higher flip
+//   EP    = EP0 + ((1 + u)^(t / 2^RC - 1) - 1) (CP + EP0)            one add per row-RC-or-higher flip
 //   Edec  = Ecol + (RC + 1) u (Cc + Ecol) + EP + (u CL + e64) + u (Cc + CL)
 //         + u CT + u (CT + CP) + u (CT + CP + CL)                  slow-path rebuild, E_L, threshold
 // (the fields and c(x_f) are FP64 sums of k terms, plus a five-level warp sum for c(x_f), each
@@ -1012,7 +1012,7 @@ double fp32_error_bound(const HostInst &h, int anchor_bits, double margin)
     const double u = std::ldexp(1.0, -24);
     const int a = std::min(std::max(anchor_bits, m.rc + 1), m.L);
     const double Ecol = m.Ecol0 + std::expm1(std::ldexp(1.0, a) * std::log1p(u)) * (m.Cc + m.Ecol0);
-    const double tP = std::ldexp(1.0, std::max(0, a - m.rc - 1)) + 1.0;
+    const double tP = std::ldexp(1.0, a - m.rc) - 1.0;  // walk steps 1 .. 2^a - 1 that flip a row >= rc
     const double EP = m.EP0 + std::expm1(tP * std::log1p(u)) * (m.CP + m.EP0);
     return Ecol + (m.rc + 1) * u * (m.Cc + Ecol) + EP + m.rest + 3.0 * u * margin;
 }

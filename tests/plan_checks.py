@@ -103,7 +103,8 @@ def fp32_bound(Q, B, L, RC, anchor_bits, margin=1e-3):
     a = min(max(anchor_bits, RC + 1), L)
     Ecol = Ecol0 + np.expm1(2.0 ** a * np.log1p(u)) * (Cc + Ecol0)
     EP0 = (u + (k + 8) * u64) * bF + (L - RC) * u * CP + (u + k * u64) * rF[B + RC:nf].sum()
-    tP = 2.0 ** max(0, a - RC - 1) + 1
+    # P takes one add at every flip of a walked row >= RC between two anchors
+    tP = sum(1 for t in range(1, 1 << a) if (t & -t).bit_length() - 1 >= RC)
     EP = EP0 + np.expm1(tP * np.log1p(u)) * (CP + EP0)
     return (Ecol + (RC + 1) * u * (Cc + Ecol) + EP + (u * CL + e64) + u * (Cc + CL) + u * CT + u * (CT + CP)
             + u * (CT + CP + CL))
