@@ -818,19 +818,20 @@ int job_enqueue_finalize(Workspace &ws, Job &j, unsigned long long max_count, un
 }
 
 // FP32 scans: the candidate margin must cover twice the measured drift plus the rounding of the
-// per-step threshold arithmetic (a few FP32 operations on values bounded by beta; the factored
-// scan's E_L plus up to 14 zero-row couplings, more).  Otherwise the caller rescans with a
+// per-step threshold arithmetic (a few FP32 operations on values bounded by beta, and by the energy
+// window where it is part of them (2 beta and more takes in every state); the factored scan's E_L plus
+// up to 14 zero-row couplings, more).  Otherwise the caller rescans with a
 // shorter walk, the dense FP32 scan, a proven margin, or FP64.  Direct evaluation sums in FP64, but
 // its records hold FP32 energies: beyond FP32's range, infinities.
 constexpr double kFp32Beta = 1e30;  // energies an FP32 scan is given
-double float_slack(Acc acc, double beta)
+double float_slack(Acc acc, double beta, double window)
 {
-    return (acc == ACC_F32Z ? 32.0 : 8.0) * std::ldexp(1.0, -24) * (1.0 + beta);
+    return std::ldexp((acc == ACC_F32Z ? 32.0 : 8.0) * (1.0 + beta) + 4.0 * std::min(std::max(0.0, window), 2.0 * beta), -24);
 }
-double scan_slack(Acc acc, const HostInst &h)
+double scan_slack(Acc acc, const HostInst &h, double window)
 {
     const bool fp32 = acc == ACC_F32 || acc == ACC_F32Z;
-    return fp32 && !(h.small && h.beta < kFp32Beta) ? float_slack(acc, h.beta) : 0.0;
+    return fp32 && !(h.small && h.beta < kFp32Beta) ? float_slack(acc, h.beta, window) : 0.0;
 }
 bool float_margin_ok(const Part &p, double margin)
 {
@@ -881,7 +882,7 @@ Part part_from(const Down &d, const Job &j, int i)
         p.candidates = d.sts[i].nrec;
         p.drift = ubits_to_double(d.sts[i].drift);
         p.err = ubits_to_double(d.sts[i].err);
-        p.slack = scan_slack(j.acc, *j.insts[i]);
+        p.slack = scan_slack(j.acc, *j.insts[i], j.window);
         p.overflow = d.sts[i].dropped > 0;
         p.dbg = d.sts[i].dbg;
     }
@@ -1003,7 +1004,8 @@ struct SolveStats {
 int solve_range(Workspace &ws, HostInst &h, int fix_bits, uint64_t fix_value, const SolveCfg &c,
                 cudaStream_t stream, Part &out, SolveStats &stats, double t_deadline)
 {
-    int st = plan_run(h, fix_bits, fix_value, c.split_k, c.walk_bits, c.variant, c.flags, c.margin);
+    int st = plan_run(h, fix_bits, fix_value, c.split_k, c.walk_bits, c.variant, c.flags, c.margin,
+                      std::max(0.0, c.window));
     if (st)
         return st;
     h.thr0 = threshold_bound(h, std::max(1, c.K));
@@ -1066,9 +1068,10 @@ int solve_proven(Workspace &ws, HostInst &h, const qubo_options &o, SolveCfg c, 
     if (st || h.acc != ACC_F32 || h.small)
         return st;
     h.anchor_bits = std::max(variant_reg_rows(h) + 1, std::min(h.anchor_bits, h.L));
-    // the bound's threshold terms carry the margin itself (a few 2^-24 of it)
-    const double m = 2.0 * fp32_error_bound(h, h.anchor_bits, c.margin) * 1.0001;
-    if (!(m > c.margin) || 2.0 * fp32_error_bound(h, h.anchor_bits, m) > m)
+    // the bound's threshold terms carry the margin itself (a few 2^-24 of it) and the window
+    const double window = std::max(0.0, c.window);
+    const double m = 2.0 * fp32_error_bound(h, h.anchor_bits, c.margin + window) * 1.0001;
+    if (!(m > c.margin) || 2.0 * fp32_error_bound(h, h.anchor_bits, m + window) > m)
         return QUBO_OK;
     c.margin = m;
     c.give_up_records = kProvenRecords;
@@ -1180,12 +1183,12 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
     int st;
     const bool fp32 = h.acc == ACC_F32 && !(c.flags & (QUBO_FLAG_PLAIN | QUBO_FLAG_RIGOROUS));
     bool done = false, tried = false;
-    if (fp32 && !(2.0 * float_slack(h.acc, h.beta) < c.margin)) {  // little or no room for a drift in the margin
+    if (fp32 && !(2.0 * float_slack(h.acc, h.beta, c.window) < c.margin)) {  // little or no room for a drift in the margin
         tried = true;
         if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
             return st;
-        if (!done && scan_slack(h.acc, h) > 0.0)
-            h.acc = float_slack(h.acc, h.beta) < c.margin ? ACC_F32 : ACC_F64;
+        if (!done && scan_slack(h.acc, h, c.window) > 0.0)
+            h.acc = float_slack(h.acc, h.beta, c.window) < c.margin ? ACC_F32 : ACC_F64;
     }
     if (!done && (st = solve_range(ws, h, o.fix_bits, o.fix_value, c, stream, p, stats, deadline)))
         return st;
@@ -1266,7 +1269,7 @@ void fill_plan_info(const HostInst &h, const SolveStats &stats, double t0, qubo_
 
 // The FP32 scan's worst-case rounding bound at the run's re-anchoring period and the longest
 // period at which it alone proves the candidates (single-instance results).
-void fill_fp32_bound(const HostInst &h, double margin, qubo_result *info)
+void fill_fp32_bound(const HostInst &h, double margin, qubo_result *info, double window = 0.0)
 {
     if (!info)
         return;
@@ -1274,8 +1277,8 @@ void fill_fp32_bound(const HostInst &h, double margin, qubo_result *info)
     info->fp32_rigorous_anchor_bits = -1;
     if (h.acc != ACC_F32 || h.small)
         return;
-    info->fp32_err_bound = fp32_error_bound(h, std::min(h.anchor_bits, h.L), margin);
-    info->fp32_rigorous_anchor_bits = fp32_rigorous_anchor_bits(h, margin);
+    info->fp32_err_bound = fp32_error_bound(h, std::min(h.anchor_bits, h.L), margin + window);
+    info->fp32_rigorous_anchor_bits = fp32_rigorous_anchor_bits(h, margin, window);
 }
 
 int batch_plan(std::vector<HostInst> &hs, int topk, std::vector<int> &order);
@@ -1817,7 +1820,7 @@ int qubo_solve_window(const void *Q_host, int n, qubo_dtype dtype, double window
         std::memset(info, 0, sizeof(*info));
     fill_outputs(h, p, 0, 0, nullptr, nullptr, nullptr, nullptr, info);
     fill_plan_info(h, stats, t0, info);
-    fill_fp32_bound(h, o.margin > 0 ? o.margin : kDefaultMargin, info);
+    fill_fp32_bound(h, o.margin > 0 ? o.margin : kDefaultMargin, info, window);
     *out_count = p.win.size();
     const size_t nw = std::min(cap, p.win.size());
     for (size_t t = 0; t < nw; ++t) {
@@ -2310,7 +2313,7 @@ int qubo_batch_fetch(qubo_batch *b, void *out_min, uint64_t *out_states, uint64_
         const InstState &sts = d.sts[r];
         const double drift = ubits_to_double(sts.drift);
         const bool fast = res.has && sts.dropped == 0 && sts.scanned == (1ull << h.n) &&
-                          (h.acc != ACC_F32 || 2.0 * drift + float_slack(h.acc, h.beta) < c.margin);
+                          (h.acc != ACC_F32 || 2.0 * drift + float_slack(h.acc, h.beta, j.window) < c.margin);
         qubo_result *inf = info ? info + i : nullptr;
         if (fast) {
             // common case: copy straight from the staging buffer

@@ -128,17 +128,18 @@ int zero_rows_search(HostInst &h);
 bool i32z_allowed();
 bool plan_factored(HostInst &h, Acc acc, int fix_bits, uint64_t fix_value, int split_k, int walk_bits);
 int plan_run(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bits, int variant_req,
-             uint32_t flags, double margin = kDefaultMargin);
+             uint32_t flags, double margin = kDefaultMargin, double window = 0.0);
 
 // Initial threshold: a bound on the K-th lowest energy of the run's sub-cube from greedy descents.
 double threshold_bound(const HostInst &h, int K, int restarts = 24);
 
 // Dense FP32 scan: worst-case rounding error of a state's decision value at a re-anchoring period
 // of 2^anchor_bits walk steps, and the longest period whose bound alone guarantees the candidates
-// (2 bound <= margin; -1 if none).  0 / -1 for other accumulators.
+// (2 bound <= margin; -1 if none).  0 / -1 for other accumulators.  mu: the candidate margin plus the
+// energy window, if any.
 const Fp32BoundTerms &fp32_bound_terms(const HostInst &h);
-double fp32_error_bound(const HostInst &h, int anchor_bits, double margin);
-int fp32_rigorous_anchor_bits(const HostInst &h, double margin);
+double fp32_error_bound(const HostInst &h, int anchor_bits, double mu);
+int fp32_rigorous_anchor_bits(const HostInst &h, double margin, double window = 0.0);
 
 }  // namespace host
 }  // namespace qubo

@@ -683,7 +683,7 @@ bool plan_factored(HostInst &h, Acc acc, int fix_bits, uint64_t fix_value, int s
 }
 
 static int plan_uncentered(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bits, int variant_req,
-                           uint32_t flags, double margin)
+                           uint32_t flags, double margin, double window)
 {
     if ((h.acc == ACC_F32 || h.acc == ACC_F32Z) && !(flags & QUBO_FLAG_PLAIN)) {
         // the rounding bound is derived for the dense FP32 scan only
@@ -699,7 +699,7 @@ static int plan_uncentered(HostInst &h, int fix_bits, uint64_t fix_value, int sp
                 return st;
             if (h.small)
                 return QUBO_OK;
-            const int a = fp32_rigorous_anchor_bits(h, margin);
+            const int a = fp32_rigorous_anchor_bits(h, margin, window);
             if (a >= 0) {
                 h.anchor_bits = std::min(h.anchor_bits, a);
                 return QUBO_OK;
@@ -753,9 +753,9 @@ static int plan_uncentered(HostInst &h, int fix_bits, uint64_t fix_value, int sp
 }
 
 int plan_run(HostInst &h, int fix_bits, uint64_t fix_value, int split_k, int walk_bits, int variant_req,
-             uint32_t flags, double margin)
+             uint32_t flags, double margin, double window)
 {
-    const int st = plan_uncentered(h, fix_bits, fix_value, split_k, walk_bits, variant_req, flags, margin);
+    const int st = plan_uncentered(h, fix_bits, fix_value, split_k, walk_bits, variant_req, flags, margin, window);
     if (st == QUBO_OK)
         center_rows(h);
     return st;
@@ -887,7 +887,8 @@ namespace host {
 //           fixed couplings w_r) and every partial sum that forms one;
 //   CL    = max_g |E_L(g)|;  bF = sum |U| within F;  rF(v) = sum_{f in F} |U_vf|;
 //   rS(r) = sum_{b in S} |U_rb|;  CabsF = sum_{b in S} rF(b);  CP = bF + sum_{r >= RC} rF(r);
-//   CT    = beta (1 + 2^-20) + margin (any threshold is a state's energy, rounded);
+//   CT    = beta (1 + 2^-20) + mu (any threshold is a state's energy, rounded), mu = the candidate margin
+//           plus the energy window, if any;
 //   e64   = n^2 2^-52 beta (error of one FP64-summed table entry before its FP32 rounding),
 //   u64   = 2^-52 (a generous FP64 rounding unit, for the per-unit fields summed in FP64),
 // the error of the decision value of any state is at most
@@ -901,14 +902,14 @@ namespace host {
 //         + (L - RC) u CP                                         each rounded once; re-anchoring
 //   EP    = EP0 + ((1 + u)^(t / 2^RC - 1) - 1) (CP + EP0)            one add per row-RC-or-higher flip
 //   Edec  = Ecol + (RC + 1) u (Cc + Ecol) + EP + (u CL + e64) + u (Cc + CL)
-//         + u CT + u (CT + CP) + u (CT + CP + CL)                  slow-path rebuild, E_L, threshold
+//         + u mu + u CT + u (CT + CP) + u (CT + CP + CL)           slow-path rebuild, E_L, threshold
 // (the fields and c(x_f) are FP64 sums of k terms, plus a five-level warp sum for c(x_f), each
 // rounded to FP32 once; lin(j) adds at most B of the rounded fields in FP32, B + 2 additions).
 // A state x of the answer has E(x) <= E(y) for the state y whose
 // computed energy set the threshold, so it is recorded whenever 2 Edec <= margin; its FP64
 // rescoring then decides.  The bound is a worst case over every state of the run.
-// The plan-dependent magnitudes of the bound, computed once per (B, L, RC) and kept in h; the margin
-// enters CT alone (three times u).
+// The plan-dependent magnitudes of the bound, computed once per (B, L, RC) and kept in h; mu enters
+// CT and its own rounding alone (four times u).
 const Fp32BoundTerms &fp32_bound_terms(const HostInst &h)
 {
     Fp32BoundTerms &m = h.fp32_terms;
@@ -1004,7 +1005,7 @@ const Fp32BoundTerms &fp32_bound_terms(const HostInst &h)
     return m;
 }
 
-double fp32_error_bound(const HostInst &h, int anchor_bits, double margin)
+double fp32_error_bound(const HostInst &h, int anchor_bits, double mu)
 {
     if (h.acc != ACC_F32 || h.small || h.Uf.empty())
         return 0.0;
@@ -1014,19 +1015,20 @@ double fp32_error_bound(const HostInst &h, int anchor_bits, double margin)
     const double Ecol = m.Ecol0 + std::expm1(std::ldexp(1.0, a) * std::log1p(u)) * (m.Cc + m.Ecol0);
     const double tP = std::ldexp(1.0, a - m.rc) - 1.0;  // walk steps 1 .. 2^a - 1 that flip a row >= rc
     const double EP = m.EP0 + std::expm1(tP * std::log1p(u)) * (m.CP + m.EP0);
-    return Ecol + (m.rc + 1) * u * (m.Cc + Ecol) + EP + m.rest + 3.0 * u * margin;
+    return Ecol + (m.rc + 1) * u * (m.Cc + Ecol) + EP + m.rest + 4.0 * u * mu;
 }
 
 // Longest re-anchoring period (log2 of walk steps, from one unrolled body up to the whole walk)
-// whose rounding bound alone guarantees the FP32 scan's candidates: 2 fp32_error_bound <= margin.
-// -1 when even one body is too long.
-int fp32_rigorous_anchor_bits(const HostInst &h, double margin)
+// whose rounding bound alone guarantees the FP32 scan's candidates: 2 fp32_error_bound <= margin, with
+// the states up to an energy window (0: none) above the minimum among them.  -1 when even one body is
+// too long.
+int fp32_rigorous_anchor_bits(const HostInst &h, double margin, double window)
 {
     if (h.acc != ACC_F32 || h.small || h.Uf.empty())
         return -1;
     const int rc = variant_reg_rows(h);
     for (int a = h.L; a >= rc + 1; --a)
-        if (2.0 * fp32_error_bound(h, a, margin) <= margin)
+        if (2.0 * fp32_error_bound(h, a, margin + window) <= margin)
             return a;
     return -1;
 }

@@ -60,14 +60,15 @@ def fp32_lanes_fit(Q, B, L, RC):
     return C + el + 1 < 2**24
 
 
-def fp32_bound(Q, B, L, RC, anchor_bits, margin=1e-3):
+def fp32_bound(Q, B, L, RC, anchor_bits, margin=1e-3, window=0.0):
     """Worst-case rounding error of the dense FP32 scan's decision value for a plan with B suffix
     bits, L walked bits (suffix = variables 0..B-1, walked = B..B+L-1, fixed = the rest), RC
     register rows, re-anchored every 2^anchor_bits walk steps: every FP32 operation rounds to
     nearest (error <= u |result|, u = 2^-24), the tables are FP64 sums rounded once, and each
     quantity's magnitude is bounded from |U| over the variables it involves (column values Cc,
     walked energies CL, prefix energy CP, thresholds CT); the per-unit fields and c(x_f) are
-    FP64 sums rounded to FP32 once, the column fields lin(j) FP32 sums of them."""
+    FP64 sums rounded to FP32 once, the column fields lin(j) FP32 sums of them; the margin plus the
+    energy window is one FP32 value, added to the threshold."""
     U = oracle.fold(np.asarray(Q, dtype=np.float64))
     n = U.shape[0]
     nf = B + L
@@ -91,7 +92,8 @@ def fp32_bound(Q, B, L, RC, anchor_bits, margin=1e-3):
     G = ((g[:, None] >> np.arange(L)) & 1).astype(np.float64)
     Uw = U[B:nf, B:nf]
     CL = np.abs(G @ np.diag(Uw) + ((G @ np.triu(Uw, 1)) * G).sum(1)).max() * (1 + 2.0 ** -30)
-    CT = beta * (1 + 2.0 ** -20) + margin
+    mu = margin + window
+    CT = beta * (1 + 2.0 ** -20) + mu
     e64 = n * n * 2.0 ** -52 * beta
     u64 = 2.0 ** -52
     Ecol0 = 2 * u * Cc + e64 + (B + 3) * u * CabsF + k * u64 * CabsF + (L - RC) * u * Cc
@@ -106,5 +108,5 @@ def fp32_bound(Q, B, L, RC, anchor_bits, margin=1e-3):
     # P takes one add at every flip of a walked row >= RC between two anchors
     tP = sum(1 for t in range(1, 1 << a) if (t & -t).bit_length() - 1 >= RC)
     EP = EP0 + np.expm1(tP * np.log1p(u)) * (CP + EP0)
-    return (Ecol + (RC + 1) * u * (Cc + Ecol) + EP + (u * CL + e64) + u * (Cc + CL) + u * CT + u * (CT + CP)
+    return (Ecol + (RC + 1) * u * (Cc + Ecol) + EP + (u * CL + e64) + u * (Cc + CL) + u * mu + u * CT + u * (CT + CP)
             + u * (CT + CP + CL))

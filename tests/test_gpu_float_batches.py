@@ -93,3 +93,21 @@ def test_entries_beyond_fp32(q, n):
         assert r.info["fp32_max_abs_err"] <= 1e-9 * abs(o.min), r.info
     b.close()
     p.close()
+
+
+@pytest.mark.parametrize("scale", [1.0, 100.0])
+def test_window_is_part_of_the_rounding_bound(q, scale):
+    """A float window's width is added to the threshold in FP32, and the bound counts the rounding of the
+    sum: reported with the run, and every state of wide and narrow windows returned."""
+    from plan_checks import fp32_bound
+
+    Q = np.random.default_rng(7).uniform(-scale, scale, (19, 19))
+    o = oracle.solve(Q, topk=4096, cap=1)
+    for k in (1, 20, 3000):
+        width = float(np.nextafter(o.topk_E[k] - o.min, np.inf))
+        sel = o.topk_E <= o.min + width
+        cnt, codes, E, info = q.solve_window(Q, width)
+        assert info["acc"] == "f32" and cnt == int(sel.sum())
+        assert np.array_equal(codes, o.topk[sel]) and np.array_equal(E, o.topk_E[sel])
+        ref = fp32_bound(Q, info["suffix_bits"], info["walk_bits"], info["reg_rows"], info["anchor_bits"], window=width)
+        assert info["fp32_err_bound"] == pytest.approx(ref, rel=1e-9)
