@@ -29,7 +29,7 @@ using namespace qubo::host;
 
 namespace {
 
-constexpr unsigned long long kDefaultRecCap = 1ull << 22;  // candidate records per job (64 MiB)
+constexpr unsigned long long kDefaultRecCap = 1ull << 22;  // candidate records per job (64 MiB, a batch's twice that)
 constexpr unsigned long long kBatchGraphRecords = 1ull << 18;  // candidate records of a replayed batch
 // Run fn(lo, hi) over [0, count) split into contiguous ranges on up to one host thread per core,
 // at least min_per_thread items per thread (small counts run on the calling thread).
@@ -458,6 +458,7 @@ struct Job {
     std::vector<size_t> off_W, off_W64, off_U64, off_Es, off_M, off_EL, off_perm;
     int max_entries = 0;
     int blocks = 0;
+    unsigned long long max_records = kDefaultRecCap;  // a power of two; a batch has as many again as scratch
     unsigned long long rec_cap = 0;
     double t_start = 0.0;
     bool aborted = false;
@@ -550,7 +551,8 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
     int st;
     if ((st = job_layout(j)))
         return st;
-    if ((st = ws.ensure(j.arena_bytes + extra_arena, kDefaultRecCap, j.up_bytes, j.down_bytes)))
+    if ((st = ws.ensure(j.arena_bytes + extra_arena, ni > 1 ? 2 * j.max_records : j.max_records, j.up_bytes,
+                        j.down_bytes)))
         return st;
     char *up = (char *)ws.h_up;
     char *dev = (char *)ws.d_arena;
@@ -654,8 +656,7 @@ int job_stage(Workspace &ws, Job &j, size_t extra_arena = 0)
             stage_one(i);
     });
     j.total_items = total;
-    // a batch's records are moved to per-instance segments in the buffer's upper half
-    j.rec_cap = std::min(ni > 1 ? ws.rec_cap / 2 : ws.rec_cap, record_capacity());
+    j.rec_cap = std::min(j.max_records, record_capacity());
     if (j.give_up_records)
         j.rec_cap = std::min(j.rec_cap, j.give_up_records);
     int &bps = ws.blocks_per_sm[{(int)j.acc, j.K <= 1, j.variant}];
@@ -898,9 +899,10 @@ int job_enqueue_finish(Workspace &ws, Job &j)
     const Down d = down_view(ws, j);
     const FinishOut o{d.hdr, d.res, d.sts, d.ties, d.tk, d.tke};
     CK(launch_finish((const Inst *)(dev + j.off_inst), (InstState *)(dev + j.off_state), ws.d_rec,
-                     ws.d_rec + ws.rec_cap / 2, (const unsigned long long *)(dev + j.off_ctr) + 1, j.rec_cap, ni,
-                     acc_float(j.acc), j.window >= 0.0, j.K, j.cap, (unsigned long long *)(dev + j.off_starts), o,
-                     j.stream, &j.launches));
+                     ni > 1 ? ws.d_rec + j.max_records : nullptr,
+                     (const unsigned long long *)(dev + j.off_ctr) + 1, j.rec_cap, ni, acc_float(j.acc),
+                     j.window >= 0.0, j.K, j.cap, (unsigned long long *)(dev + j.off_starts), o, j.stream,
+                     &j.launches));
     CK(record_event(ws.ev[2], j.stream));
     return QUBO_OK;
 }
@@ -2212,14 +2214,14 @@ int qubo_batch_create(const void *Q_packed, const int *n, const size_t *offsets,
     j.cap = states_cap_per_inst;
     j.margin = kDefaultMargin;
     j.variant = b->hs[0].variant;
+    // Batches produce few candidates per instance (an instance that overflows the buffer is solved again
+    // on its own at fetch time).
+    j.max_records = kBatchGraphRecords;
     // the initial per-instance state lives after the job's arena and is copied in at every run
     // (with the counters behind it)
     if ((st = job_stage(b->ws, j, align_up(sizeof(InstState) * (size_t)count, 256) + 512)))
         return st;
     const size_t state_bytes = j.off_items - j.off_state;
-    // Batches produce few candidates per instance (an instance that overflows the buffer is solved again
-    // on its own at fetch time).
-    j.rec_cap = std::min<unsigned long long>(j.rec_cap, kBatchGraphRecords);
     b->off_state_init = align_up(j.arena_bytes, 256);
     char *dev_arena = (char *)b->ws.d_arena;
     CK(cudaMemcpy(dev_arena, b->ws.h_up, j.up_bytes, cudaMemcpyHostToDevice));

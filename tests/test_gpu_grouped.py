@@ -266,3 +266,13 @@ def test_two_limbs_longest_walk(q, walk, tmp_path):
         assert r.info["acc"] == "i64" and r.info["grouped"] == 1, r.info
         assert r.info["walk_bits"] == walk if walk <= 14 else r.info["walk_bits"] <= 14, r.info
         check(r, oracle.solve(Q, topk=3, cap=64))
+
+
+def test_a_batch_has_the_whole_record_buffer(q):
+    """2^21 minimisers and a little more in one batch, half of what the buffer of a call holds: no
+    instance is solved a second time."""
+    Qs = [wl.diagonal(22, seed=3, zeros=21)] + [wl.upper_int(17, -50, 50, seed=9 + k) for k in range(3)]
+    rs = q.solve_batched(Qs, topk=4)
+    assert rs[0].n_ties == 1 << 21 and rs[0].info["passes"] == 1, rs[0].info
+    for Q, r in list(zip(Qs, rs))[1:]:
+        check(r, oracle.solve(Q, topk=4, cap=64))
