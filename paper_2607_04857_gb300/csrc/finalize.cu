@@ -300,6 +300,8 @@ __global__ void extract_kernel(const Rec *rec, bool batched, int n_inst, int top
 // the general path (FinishOut::hdr, ResOut::has = 2).  A batch's records, interleaved in the buffer,
 // are first moved to one segment per instance.  Latency-bound throughout.
 
+constexpr unsigned long long kLongList = ~0ull;  // cursor of a list that finish_kernel leaves alone
+
 // Exclusive sums of the stored records per instance (one block).
 __global__ void __launch_bounds__(1024) segment_kernel(const InstState *state, int n_inst, unsigned long long *starts,
                                                        unsigned long long *cursor)
@@ -336,7 +338,7 @@ __global__ void __launch_bounds__(1024) segment_kernel(const InstState *state, i
         const unsigned long long excl = carry + (warp ? warp_sums[warp - 1] : 0ull) + sum - c;
         if (i < n_inst) {
             starts[i] = excl;
-            cursor[i] = excl;
+            cursor[i] = c > (unsigned long long)kChunk ? kLongList : excl;
         }
         __syncthreads();
         if (threadIdx.x == 1023)
@@ -347,7 +349,8 @@ __global__ void __launch_bounds__(1024) segment_kernel(const InstState *state, i
         starts[n_inst] = carry;
 }
 
-// Move every record to its instance's segment; float records are rescored on the way.
+// Move every record of a list that finish_kernel sorts to its instance's segment; float records are
+// rescored on the way.  The records of a longer list stay: the general path rescores and sorts those.
 template <bool FL>
 __global__ void scatter_kernel(const Inst *insts, InstState *state, const Rec *rec, const unsigned long long *d_nrec,
                                unsigned long long cap, int n_inst, unsigned long long *cursor, Rec *out)
@@ -357,7 +360,7 @@ __global__ void scatter_kernel(const Inst *insts, InstState *state, const Rec *r
          i += (unsigned long long)gridDim.x * blockDim.x) {
         Rec r = rec[i];
         const uint64_t inst = rec_inst(r.key, true);
-        if (inst >= (uint64_t)n_inst)
+        if (inst >= (uint64_t)n_inst || __ldcg(cursor + inst) == kLongList)
             continue;
         if constexpr (FL) {
             const double e64 = energy_fp64(insts[inst].U64, insts[inst].n, rec_code(r.key, true));
@@ -480,7 +483,8 @@ cudaError_t launch_finish(const Inst *d_inst, InstState *d_state, Rec *rec, Rec 
     if (batched) {
         unsigned long long *cursor = d_starts + n_inst + 1;
         segment_kernel<<<1, 1024, 0, s>>>(d_state, n_inst, d_starts, cursor);
-        const int blocks = n_inst < 65536 ? (n_inst + 15) / 16 : 4096;  // a few records per instance
+        // a few records per instance as a rule, but a small batch's lists may hold 2048 each
+        const int blocks = n_inst < 1024 ? 64 : (n_inst + 15) / 16;
         if (is_float)
             scatter_kernel<true><<<blocks, 256, 0, s>>>(d_inst, d_state, rec, d_nrec, cap, n_inst, cursor, segments);
         else
