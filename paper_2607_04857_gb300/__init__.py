@@ -178,9 +178,11 @@ def _stream_ptr(stream):
     """cudaStream_t as an integer: an int, an object with .cuda_stream (torch), or the current
     torch stream when torch with CUDA is in use; else the default stream."""
     if stream is None:
-        torch = sys.modules.get("torch")  # a process that has not imported it has no current torch stream
-        if torch is not None and torch.cuda.is_initialized():
-            return int(torch.cuda.current_stream().cuda_stream)
+        # a process that has not imported torch (or is at it, in another thread) has no current torch stream
+        cuda = getattr(sys.modules.get("torch"), "cuda", None)
+        initialized = getattr(cuda, "is_initialized", None)
+        if initialized is not None and initialized():
+            return int(cuda.current_stream().cuda_stream)
         return None
     if hasattr(stream, "cuda_stream"):
         return int(stream.cuda_stream)

@@ -205,3 +205,18 @@ def test_merge_rejects_inputs_whose_counts_exceed_their_arrays(q):
                     dict(n_written=2, n_ties=1)):
             assert merge(ctypes.byref(good), ctypes.byref(part(cls, **bad)), 4, 0, ctypes.byref(out)) == \
                 q.QUBO_ERR_ARG, bad
+
+
+def test_default_stream_while_torch_is_being_imported(q, monkeypatch):
+    """Another thread importing torch leaves modules without their later attributes in sys.modules."""
+    import sys
+    import types
+
+    torch = types.ModuleType("torch")
+    monkeypatch.setitem(sys.modules, "torch", torch)
+    assert q._stream_ptr(None) is None
+    torch.cuda = types.ModuleType("torch.cuda")
+    assert q._stream_ptr(None) is None
+    torch.cuda.is_initialized = lambda: True
+    torch.cuda.current_stream = lambda: types.SimpleNamespace(cuda_stream=7)
+    assert q._stream_ptr(None) == 7
