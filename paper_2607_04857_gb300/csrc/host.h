@@ -86,7 +86,7 @@ struct PlanFields {
     Acc acc;
     int variant, B, L, k, small, fix_bits;
     uint64_t fix_value, unit_begin, units, sub_base, sub_count, items, states;
-    int32_t clampC, col_lo, col_hi, el_fused, elmin, group_ok;
+    int32_t clampC, col_lo, col_hi, el_fused, elmin, group_ok, center[4];
 };
 
 // Plans, saved and restored without the matrices.

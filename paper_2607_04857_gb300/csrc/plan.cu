@@ -25,7 +25,7 @@ PlanFields plan_fields(const HostInst &h)
 {
     return {h.acc,   h.variant,  h.B,         h.L,     h.k,      h.small,  h.fix_bits, h.fix_value, h.unit_begin,
             h.units, h.sub_base, h.sub_count, h.items, h.states, h.clampC, h.col_lo,   h.col_hi,    h.el_fused,
-            h.elmin, h.group_ok};
+            h.elmin, h.group_ok, {h.center[0], h.center[1], h.center[2], h.center[3]}};
 }
 
 void set_plan_fields(HostInst &h, const PlanFields &p)
@@ -50,8 +50,7 @@ void set_plan_fields(HostInst &h, const PlanFields &p)
     h.el_fused = p.el_fused;
     h.elmin = p.elmin;
     h.group_ok = p.group_ok;
-    for (int32_t &c : h.center)
-        c = 0;
+    std::copy(p.center, p.center + 4, h.center);
 }
 
 bool dtype_ok(qubo_dtype dt) { return dt == QUBO_I16 || dt == QUBO_I32 || dt == QUBO_F32 || dt == QUBO_F64; }

@@ -164,3 +164,47 @@ def test_fp32_rigorous_period_of_the_benchmark_instance(q):
     assert p["walk_bits"] == 14 and p["anchor_bits"] == 10
     assert 2 * p["fp32_err_bound"] > 1e-3
     assert p["fp32_rigorous_anchor_bits"] == 6
+
+
+def test_a_restored_plan_is_the_plan_that_was_saved(q, tmp_path):
+    """The batch autotuner saves a plan, tries another and restores it: the mean moves of E_L that the
+    grouped scan keeps in its rows (center_rows) come back with it, for all later trials' times."""
+    import os
+    import subprocess
+
+    pkg = os.path.dirname(q.LIB_PATH)
+    src = tmp_path / "plans.cpp"
+    src.write_text("""
+#include "host.h"
+using namespace qubo;
+using namespace qubo::host;
+int main()
+{
+    const int n = 26;
+    std::vector<int32_t> Q(n * n, 0);
+    for (int i = 0; i < n; ++i)
+        for (int j = i; j < n; ++j)
+            Q[i * n + j] = i == j ? -13 : 1;  // Max-Cut of the complete graph, halved
+    HostInst h;
+    if (prepare(Q.data(), n, QUBO_I32, 0, h) || plan_run(h, 0, 0, 0, 9, -1, 0))
+        return 1;
+    if (!grouped_form(h.acc, h.variant) || h.center[0] == 0)
+        return 2;
+    const HostInst before = h;
+    const PlanFields saved = plan_fields(h);
+    if (plan(h, 0, 0, 0, 8))
+        return 3;
+    for (int32_t &c : h.center)
+        c = 99;
+    set_plan_fields(h, saved);
+    for (int r = 0; r < 4; ++r)
+        if (h.center[r] != before.center[r])
+            return 4;
+    return h.L == before.L && h.acc == before.acc && h.variant == before.variant ? 0 : 5;
+}
+""")
+    exe = str(tmp_path / "plans")
+    inc = [os.path.join(pkg, "csrc"), os.path.join(os.path.dirname(pkg), "include"), "/usr/local/cuda/include"]
+    subprocess.run(["g++", "-std=c++20", *(x for i in inc for x in ("-I", i)), str(src), q.LIB_PATH,
+                    "-Wl,-rpath," + pkg, "-o", exe], check=True)
+    assert subprocess.run([exe]).returncode == 0
