@@ -740,10 +740,11 @@ static int plan_uncentered(HostInst &h, int fix_bits, uint64_t fix_value, int sp
         h.variant = pick_variant(h.acc, variant_req);
         h.variant = fit_variant(h, fix_bits, split_k, walk_bits, variant_req, h.variant);
     } else {
-        // the two-limb kernel where its walk (at least five bits) fits
+        // the two-limb kernel where its walk (at least five bits) fits; a smaller range keeps the plain
+        // kernel's plan, and its refusal of a walk that does not fit
         const int bits = h.n - fix_bits - acc_suffix_bits(h.acc, 0);
         const int L = split_k > 0 ? h.n - acc_suffix_bits(h.acc, 0) - split_k : walk_bits > 0 ? walk_bits : bits;
-        h.variant = h.acc == ACC_I64 && L >= 5 && L <= (split_k > 0 || walk_bits > 0 ? kLimbMaxWalkBits : L) &&
+        h.variant = h.acc == ACC_I64 && bits >= 5 && L >= 5 && L <= (split_k > 0 || walk_bits > 0 ? kLimbMaxWalkBits : L) &&
                             limb_shift(h) > 0 ? kLimbVariant : 0;
     }
     if (h.acc == ACC_I16P)

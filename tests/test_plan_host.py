@@ -208,3 +208,17 @@ int main()
     subprocess.run(["g++", "-std=c++20", *(x for i in inc for x in ("-I", i)), str(src), q.LIB_PATH,
                     "-Wl,-rpath," + pkg, "-o", exe], check=True)
     assert subprocess.run([exe]).returncode == 0
+
+
+@pytest.mark.parametrize("n", [12, 13, 14])
+def test_int64_walks_that_do_not_fit_are_refused(q, n):
+    """Twelve variables are evaluated directly whatever walk is asked for; from thirteen on a walk longer
+    than the variables beside the suffix's nine is an error, as for the plain kernel."""
+    Q = wl.upper_int(n, -(1 << 30), 1 << 30, seed=n)
+    for walk in (5, 6, 12):
+        for plain in (False, True):
+            if n > 12 and walk > n - 9:
+                with pytest.raises(q.QuboError):
+                    q.plan_query(Q, walk_bits=walk, plain=plain)
+            else:
+                assert q.plan_query(Q, walk_bits=walk, plain=plain)["acc"] == "i64"
