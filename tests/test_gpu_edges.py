@@ -76,7 +76,8 @@ def test_abort_from_another_thread(q):
 
 
 def test_wide_time_limit(q):
-    """Four sub-problems of 2^42 states (about 1 s in all) under a 0.3 s limit."""
+    """Four sub-problems of 2^42 states (about 0.5 s in all in the interleaved packed scan, which wide
+    solves keep under a limit) under a 0.3 s limit."""
     Q = wl.upper_int(70, -100, 100, seed=3)
     with pytest.raises(q.QuboError) as e:
         q.solve_wide(Q, 42, outer_begin=0, outer_count=4, time_limit=0.3)

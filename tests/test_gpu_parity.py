@@ -394,7 +394,8 @@ def test_grouped_form_parity(q, lim, monkeypatch):
     over the columns while a lower bound proves they hold no candidate.  Entries from tie-heavy
     (+-3, most groups reach the threshold, many ties) to the FP32-lane limit (the bound's sum
     rounded down near 2^24; the largest entries leave the FP32 lanes for the int32 kernel, which
-    has no grouped form); top-16, K = 1 and the tie set against the oracle."""
+    keeps the interleaved form on a walk this short set by the caller); top-16, K = 1 and the tie
+    set against the oracle."""
     for k, v in LANES["i32f"].items():
         monkeypatch.setenv(k, v)
     for n, seed in ((27, 120 + lim % 7), (29, 121)):

@@ -1,9 +1,11 @@
 """The lower bound behind the grouped step form, restated in numpy and checked by brute force (no
-GPU).  A unit's columns are walked in reflected Gray order; at each group's first state the
-thread's exact column minimum m is taken, and over the group's next 15 steps (register rows 0-3)
-the minimum must never fall below m + D, where D is the smallest running sum of each step's
-smallest column move.  E_L's group minimum completes the test.  A wrong sign pattern, a dropped
-coupling to the fixed bits or a running sum taken over the wrong steps fails these checks."""
+GPU).  A unit's columns are walked in reflected Gray order in groups of 16 states, over which a
+column takes its value with the register rows 0-3 clear plus every subset of the four.  First test:
+with m the thread's exact column minimum at the group's first state and D the smallest of its
+columns' offsets (the rows' negative parts, less row 3 where the group starts with it set), no
+column falls below m + D.  Second test: each column with its own offset, the exact minimum.  E_L's
+group minimum completes both.  A wrong sign pattern, a dropped coupling to the fixed bits or an
+offset of the wrong parity fails these checks."""
 import os
 import subprocess
 
@@ -40,17 +42,11 @@ def columns_over_walk(U, B, L, fixed):
     return col, el, S
 
 
-def group_bound(M, w, par):
-    """D for one thread's columns: register rows r = 0..3 move column j by +-(M[r, j] + w[r])."""
-    lo = (M + w[:, None]).min(axis=1)
-    hi = (M + w[:, None]).max(axis=1)
-    cum, best = 0, 0
-    for t in range(1, 16):
-        kk = (t & -t).bit_length() - 1
-        neg = bool(par) if kk == 3 else bool((t >> (kk + 1)) & 1)
-        cum += -hi[kk] if neg else lo[kk]
-        best = min(best, cum)
-    return best
+def offsets(M, w, par):
+    """A column's group minimum less its value at the group's first state: register rows r = 0..3 move
+    column j by +-(M[r, j] + w[r]), and groups of odd index start with row 3 set."""
+    rows = M + w[:, None]
+    return np.minimum(rows, 0).sum(axis=0) - (rows[3] if par else 0)
 
 
 @pytest.mark.parametrize("seed", range(4))
@@ -76,25 +72,27 @@ def test_group_bound_holds_by_brute_force(seed):
             sign = -1 if (i >> (kk + 1)) & 1 else 1
             assert np.array_equal(col[i] - col[i - 1], sign * (M[kk] + w[kk]))
     for g in range(col.shape[0] // 16):
-        m = col[16 * g].min()
-        D = group_bound(M, w, g & 1)
-        assert m + D <= col[16 * g:16 * g + 16].min()
+        group, off = col[16 * g:16 * g + 16], offsets(M, w, g & 1)
+        assert np.array_equal(group[0] + off, group.min(axis=0))  # the second test
+        m, D = group[0].min(), off.min()  # the first
+        assert m + D <= group.min()
         # the test: no state of the group is at or below u when m + D > u - min E_L
-        emin = (col[16 * g:16 * g + 16] + el[16 * g:16 * g + 16, None]).min()
+        emin = (group + el[16 * g:16 * g + 16, None]).min()
         assert m + D + el[16 * g:16 * g + 16].min() <= emin
 
 
 def test_group_bound_is_tight_for_one_column():
-    """With a single column every step's smallest move is the move itself, so m + D is the
-    column's exact minimum over the group."""
+    """With a single column m + D is the column's exact minimum over the group, for either sign of
+    row 3."""
     M = np.array([[5], [-7], [3], [-2]])
     w = np.array([1, 2, -4, 0])
-    walk = [0]
-    for t in range(1, 16):
-        kk = (t & -t).bit_length() - 1
-        neg = (t >> (kk + 1)) & 1  # group 0: the sign of row 3 follows bit 4 of the position (0)
-        walk.append(walk[-1] + (-1 if neg else 1) * (M[kk, 0] + w[kk]))
-    assert group_bound(M, w, 0) == min(walk)
+    for par in (0, 1):
+        walk = [0]
+        for t in range(1, 16):
+            kk = (t & -t).bit_length() - 1
+            neg = par if kk == 3 else (t >> (kk + 1)) & 1
+            walk.append(walk[-1] + (-1 if neg else 1) * (M[kk, 0] + w[kk]))
+        assert offsets(M, w, par).min() == min(walk)
 
 
 @pytest.mark.parametrize("seed", range(3))
@@ -120,16 +118,14 @@ def test_exact_group_minimum(seed):
 def test_smallest_offset_bounds_every_column(seed):
     """The first test's bound: m + D, D the smallest over a thread's columns of the offset between a
     column's group minimum and its value at the group's first state, is at or below every column in the
-    group and at least as tight as the running sums of extreme moves."""
+    group."""
     rng = np.random.default_rng(100 + seed)
     rows, start = rng.integers(-80, 81, size=(4, 16)), rng.integers(-400, 400, size=16)
-    neg = np.minimum(rows, 0).sum(axis=0)
     for par in (0, 1):
         first = start + par * rows[3]
-        D = (neg - par * rows[3]).min()
+        D = offsets(rows, np.zeros(4, dtype=np.int64), par).min()
         least = min((start + sum(((p >> r) & 1) * rows[r] for r in range(4))).min() for p in range(16))
         assert first.min() + D <= least
-        assert D >= group_bound(rows, np.zeros(4, dtype=np.int64), par)
 
 
 def test_kept_rows_add_without_signed_overflow(tmp_path):
