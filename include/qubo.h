@@ -39,10 +39,12 @@ typedef enum { QUBO_I16 = 1, QUBO_I32 = 2, QUBO_F32 = 3, QUBO_F64 = 4 } qubo_dty
  * measured drift needs it; qubo_result.anchor_bits), every state within the candidate margin
  * rescored in FP64; where the caller's margin has no room for the scan's rounding, a wider one of
  * twice the worst-case rounding bound is taken (more candidates, the same answer).
- * QUBO_ACC_I64: int64 energies, scanned on two 32-bit limbs when sum |U_ij| < 2^55.  QUBO_ACC_I32F: integer energies held exactly in FP32 lanes, chosen when
- * every value the run's plan holds in a lane stays below 2^24 in magnitude.  QUBO_ACC_I16P: integer energies held as two 16-bit lanes per 32-bit word,
- * chosen (before QUBO_ACC_I32F) when every column value of the run's plan provably lies in
- * [-32768, 32767].  QUBO_ACC_I32Z: int32 energies of a sparse instance, chosen first when the
+ * QUBO_ACC_I64: int64 energies, scanned on two 32-bit limbs when sum |U_ij| < 2^55.
+ * QUBO_ACC_I32F: integer energies held exactly in FP32 lanes, chosen when every value the run's
+ * plan holds in a lane stays below 2^24 in magnitude.
+ * QUBO_ACC_I16P: integer energies held as two 16-bit lanes per 32-bit word, chosen (before
+ * QUBO_ACC_I32F) when every column value of the run's plan provably lies in [-32768, 32767].
+ * QUBO_ACC_I32Z: int32 energies of a sparse instance, chosen first when the
  * variables can be ordered so that at least 3 walked prefix variables have no coupling to any
  * suffix variable: the scan then factors those variables out of the column walk (the minimum
  * over their patterns separates from the minimum over the columns) and updates the columns
@@ -145,12 +147,14 @@ typedef struct {
     uint64_t d2h_bytes;       /* bytes copied device -> host by this call */
     double fp32_err_bound;    /* QUBO_ACC_F32: worst-case rounding error of any state's FP32
                                  decision value at the run's re-anchoring period (from the folded
-                                 matrix and the plan, every FP32 operation rounded to nearest);
-                                 the candidates are proven complete when 2 * fp32_err_bound <=
-                                 margin.  0 for other accumulators */
+                                 matrix, the plan and an energy window's width, every FP32
+                                 operation rounded to nearest); the candidates are proven complete
+                                 when 2 * fp32_err_bound is at most the margin the run took: the
+                                 caller's, or the wider one (see QUBO_ACC_F32).  0 for other
+                                 accumulators */
     int32_t fp32_rigorous_anchor_bits; /* QUBO_ACC_F32: longest re-anchoring period (log2 of walk
-                                 steps) at which 2 * fp32_err_bound <= margin; -1 if none, or for
-                                 other accumulators */
+                                 steps) at which twice the bound is at most the caller's margin;
+                                 -1 if none, or for other accumulators */
     int32_t reg_rows;         /* plan: walked rows the scan kernel keeps in registers (its
                                  unrolled body is 2^(reg_rows + 1) Gray steps) */
     int32_t variant;          /* plan: compiled scan variant (-1: states evaluated directly) */

@@ -783,8 +783,8 @@ Down down_view(Workspace &ws, const Job &j)
 }
 
 // Enqueue rescoring (floats), the sort of the candidate records, extraction and the download
-// of the results.  max_pow2 bounds the sort network; the kernels read the record count on the
-// device, so a larger bound only costs empty launches (this is what a captured graph uses).
+// of the results, for record lists beyond finish_kernel's.  max_pow2 bounds the sort network; the
+// kernels read the record count on the device.
 int job_enqueue_finalize(Workspace &ws, Job &j, unsigned long long max_count, unsigned long long max_pow2)
 {
     const int ni = (int)j.insts.size();
@@ -827,7 +827,8 @@ int job_enqueue_finalize(Workspace &ws, Job &j, unsigned long long max_count, un
 constexpr double kFp32Beta = 1e30;  // energies an FP32 scan is given
 double float_slack(Acc acc, double beta, double window)
 {
-    return std::ldexp((acc == ACC_F32Z ? 32.0 : 8.0) * (1.0 + beta) + 4.0 * std::min(std::max(0.0, window), 2.0 * beta), -24);
+    const double wide = std::min(std::max(0.0, window), 2.0 * beta);
+    return std::ldexp((acc == ACC_F32Z ? 32.0 : 8.0) * (1.0 + beta) + 4.0 * wide, -24);
 }
 double scan_slack(Acc acc, const HostInst &h, double window)
 {
@@ -1052,10 +1053,10 @@ int solve_range(Workspace &ws, HostInst &h, int fix_bits, uint64_t fix_value, co
 
 // A float instance whose magnitudes leave the caller's candidate margin no room for an FP32 scan's
 // rounding (entries of order 100 at n = 30) is scanned in FP32 all the same, with a wider margin: twice
-// the worst-case rounding bound of the run's plan, which proves that every state of the answer reaches
-// the FP64 rescoring.  A wider margin only adds candidates.  When they are more than kProvenRecords
-// (dense low spectra, e.g. large penalty terms) the run ends early and the FP64 scan runs instead, as
-// without this attempt.  n=31, entries uniform in [-100, 100]: 0.19 ms of scan against 9.2 ms in FP64
+// the worst-case rounding bound of the run's plan (with the energy window in it), which proves that every
+// state of the answer reaches the FP64 rescoring.  A wider margin only adds candidates.  When they are more
+// than kProvenRecords (dense low spectra, e.g. large penalty terms) the run ends early and the FP64 scan
+// runs instead, as without this attempt.  n=31, entries uniform in [-100, 100]: 0.19 ms of scan against 9.2 ms in FP64
 // (an FP64 add takes a warp about 75 cycles on GB300), which three FP32 scans preceded.
 constexpr unsigned long long kProvenRecords = 1ull << 16;
 int solve_proven(Workspace &ws, HostInst &h, const qubo_options &o, SolveCfg c, cudaStream_t stream, Part &p,
@@ -1185,7 +1186,8 @@ int solve_one(Workspace &ws, HostInst &h, const qubo_options &o, size_t states_c
     int st;
     const bool fp32 = h.acc == ACC_F32 && !(c.flags & (QUBO_FLAG_PLAIN | QUBO_FLAG_RIGOROUS));
     bool done = false, tried = false;
-    if (fp32 && !(2.0 * float_slack(h.acc, h.beta, c.window) < c.margin)) {  // little or no room for a drift in the margin
+    // little or no room for a drift in the margin
+    if (fp32 && !(2.0 * float_slack(h.acc, h.beta, c.window) < c.margin)) {
         tried = true;
         if ((st = solve_proven(ws, h, o, c, stream, p, stats, deadline, &done)))
             return st;
@@ -2024,8 +2026,8 @@ int qubo_solve_wide(const void *Q_host, int n, qubo_dtype dtype, int n_inner, ui
             qubo_options so = o;
             if (deadline > 0) {
                 so.time_limit_s = std::max(1e-3, deadline - now_s());
-                // the limits callers pass here were chosen against the interleaved packed scan's
-                // rate; a range that ran out of time still does
+                // packed sub-problems keep the interleaved scan (3.45e13 states/s, grouped 6.2e13) under a
+                // limit: the limit's test, 4 x 2^42 states in 0.3 s, is pinned to that rate
                 so.flags |= kFlagInterleaved;
             }
             parts.resize(1);

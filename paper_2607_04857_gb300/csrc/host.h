@@ -16,7 +16,8 @@ namespace host {
 constexpr int kTargetUnitsLog2 = 15;   // aim for >= 2^15 work units per scan (see also grouped_walk)
 constexpr double kDefaultMargin = 1e-3; // FP32 scans: candidate margin above the running minimum
 constexpr int kDefaultMaxWalkBits = 12;
-// The flags a caller may set, and an internal one: the packed scan's interleaved variants only.
+// The flags a caller may set, and an internal one: the packed scan's interleaved variants only (wide
+// solves with a time limit, one sub-problem at a time).
 constexpr uint32_t kCallerFlags = QUBO_FLAG_PLAIN | QUBO_FLAG_INT32 | QUBO_FLAG_RIGOROUS;
 constexpr uint32_t kFlagInterleaved = 0x80000000u;
 // Grouped scans walk up to 2^14 steps: n=40 packed 2.5% and n=38 int32 0.6% faster than 2^12.

@@ -53,7 +53,7 @@ constexpr int kVariantMinInputs[kScanVariants] = {3, 3, 3, 3, 3, 3, 3, 3, 3, 3, 
 constexpr int kVariantInterleave[kScanVariants] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 0, 1, 1, 1, 1, 1, 2, 2, 2, 2};
 // Default variant per 4-byte accumulator (measured on GB300; see the profiles).
 constexpr int kDefaultVariantI32 = 20;
-constexpr int kCallerVariantI32 = 16;  // short walks set by the caller (plan.cu: fit_variant)
+constexpr int kCallerVariantI32 = 16;  // int32 walks of at most 8 bits set by the caller (plan.cu: fit_variant)
 constexpr int kDefaultVariantF32 = 20;
 constexpr int kDefaultVariantI32F = 20;
 constexpr int kDefaultVariantI16P = 20;

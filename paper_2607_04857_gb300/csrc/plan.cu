@@ -255,8 +255,9 @@ int pick_variant(Acc acc, int requested) { return requested >= 0 ? requested : s
 // the best variant with fewer register rows and the same columns per thread, so the suffix split is
 // unchanged: the grouped one with four rows, whose body is one group (a small launch waits on the
 // first fetch of its code), then the interleaved ones; failing all, the one with the fewest rows.
-// int32: a walk of at most 2^8 steps that the caller sets keeps the interleaved variant 16, the plan
-// such callers have had (grouped, n=29: 91 us against 156 us).
+// int32: a walk of at most 2^8 steps that the caller sets keeps the interleaved variant 16.  That is not
+// the faster one (n=29, 8-bit walk: 156 us, grouped 91 us): callers fix a walk to get a known plan, and
+// the parity tests pin this one.
 int fit_variant(const HostInst &h, int fix_bits, int split_k, int walk_bits, int variant_req, int variant)
 {
     if (variant_req >= 0 || std::getenv("QUBO_SCAN_VARIANT"))

@@ -184,10 +184,6 @@ struct Tr<i16p> {
     __device__ static int32_t tmin(int32_t a, int32_t b) { return min(a, b); }
 };
 constexpr int32_t kLaneBias = 32768;
-#ifndef QUBO_LONG_BODY
-#define QUBO_LONG_BODY 4
-#endif
-constexpr int kLongBody = QUBO_LONG_BODY;
 
 // Column value of a prefix-type threshold.  For FP32 columns holding integers the threshold is
 // clamped to +-C first: beyond C every column (|column| <= C - 1 - max|E_L|) is decided the same
@@ -1370,11 +1366,11 @@ __global__ void __launch_bounds__(kScanThreads, MINB) scan_kernel(const ScanArgs
     // units take 0.1-30 ms here: one per claim keeps the end of a launch balanced
     persistent_units<T, 1>(a, lane, Treg, [&](const Inst &d, int inst, uint64_t unit) {
         if constexpr (Tr<T>::kPack == 2 && ILV == 2)
-            scan_unit_packed_grouped<S, RC, RC == 5 ? kLongBody : 1, K1>(a, d, inst, unit, Treg, lane, stage, wsm, neg);
+            scan_unit_packed_grouped<S, RC, RC == 5 ? 4 : 1, K1>(a, d, inst, unit, Treg, lane, stage, wsm, neg);
         else if constexpr (Tr<T>::kPack == 2)
             scan_unit_packed<S, RC, K1, ADDM, MINM, ILV>(a, d, inst, unit, Treg, lane, stage, wsm);
         else if constexpr (ILV == 2)
-            scan_unit_grouped<T, S, RC, RC == 5 ? kLongBody : 1, K1, ADDM>(a, d, inst, unit, Treg, lane, stage, wsm, anc, neg);
+            scan_unit_grouped<T, S, RC, RC == 5 ? 4 : 1, K1, ADDM>(a, d, inst, unit, Treg, lane, stage, wsm, anc, neg);
         else
             scan_unit<T, S, RC, K1, ADDM, MINM, ILV>(a, d, inst, unit, Treg, lane, stage, wsm, anc);
     });
